@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -47,8 +48,13 @@ struct KernelPlan {          // job list and parameter vectors of one tile-kerne
   int n_jobs = 0;
   int job_mat[kMaxJobs] = {0};
   int job_acc[kMaxJobs] = {0};
+  int job_bias[kMaxJobs] = {0};     // 1-based bias tile a job's D starts from, 0: none
+  bool folded = false;              // gamma folded into the weights, but for the MLP's last layer
   std::vector<float> vecs;
-  float* d_vecs = nullptr;
+  std::vector<const float*> biases; // the bias tiles' vectors, while the plan is made
+  float* d_vecs = nullptr;          // vecs, and behind them the ones tile and the bias tiles
+  uint8_t* d_consts = nullptr;
+  uint32_t const_bytes = 0;
   const uint8_t* wmats = nullptr;   // its weight matrices (null: the context's)
 };
 
@@ -142,6 +148,23 @@ void pack_block(const float* W, int ld, int col0, int H, bool with_lo, uint8_t* 
     }
 }
 
+// Pack a first layer's W [H, n_in], n_in <= 32, as an input matrix: its hi, mid and lo bf16 parts (fp32
+// model) or its one part (bf16 model) at their places in a weight block of zeros.
+void pack_input(const float* W, int n_in, int H, bool bf, uint8_t* out, size_t bytes) {
+  std::memset(out, 0, bytes);
+  for (int n = 0; n < H; ++n)
+    for (int k = 0; k < n_in; ++k) {
+      float v = W[(size_t)n * n_in + k];
+      for (int w = 0; w < (bf ? 1 : 3); ++w) {
+        const uint16_t part = f32_to_bf16_rne(v);
+        // parts 0 and 1 share a 64-column chunk (columns 32 w + k); part 2 starts one of its own
+        const size_t base = w < 2 ? 0 : (H == 128 ? input_part_offset<128>(2) : input_part_offset<64>(2));
+        std::memcpy(out + base + swizzled_offset(H, n, (w < 2 ? 32 * w : 0) + k), &part, 2);
+        v -= bf16_to_f32(part);
+      }
+    }
+}
+
 void push(std::vector<float>& v, const float* p, size_t n) { v.insert(v.end(), p, p + n); }
 
 // W' = (I - 11^T/H) W and b' = b - mean(b): the LayerNorm after the layer then sees a
@@ -159,6 +182,88 @@ void centre_layer(const float* W, const float* b, int H, int in, std::vector<flo
   for (int n = 0; n < H; ++n) mb += b[n];
   mb /= H;
   for (int n = 0; n < H; ++n) bc[n] = (float)(b[n] - mb);
+}
+
+// LayerNorm vectors of one layer, as the kernels read them: gamma, beta.
+void push_ln(std::vector<float>& v, const Layer& l, int H) {
+  push(v, l.g, H);
+  push(v, l.be, H);
+}
+
+// fp32 model: y_l = relu(gamma n + beta) of a hidden layer l < L equals |gamma| relu(s n + beta / |gamma|)
+// with s = sign(gamma), so the kernels need no gamma when W_l's rows and b_l carry s and W_{l+1}'s columns
+// carry |gamma| (a LayerNorm's variance does not see the sign, and the fp32 model's kernels compute no mean).  One
+// vector less is read and one multiplication less made per element of every hidden layer.  Only for
+// |gamma| in [2^-6, 2^6], where the scaling cannot overflow or lose a column; otherwise the MLP keeps
+// its gammas (false).  `lay` points at copies of the model's arrays.
+bool fold_gamma(std::vector<std::vector<float>*> W, std::vector<std::vector<float>*> b,
+                std::vector<std::vector<float>*> g, std::vector<std::vector<float>*> be, const int* in, int H) {
+  const int L = (int)W.size();
+  for (int l = 0; l + 1 < L; ++l)
+    for (int i = 0; i < H; ++i) {
+      const float a = std::fabs((*g[l])[i]);
+      if (!(a >= 0.015625f && a <= 64.f)) return false;
+    }
+  for (int l = 0; l + 1 < L; ++l)
+    for (int i = 0; i < H; ++i) {
+      const float s = (*g[l])[i] < 0.f ? -1.f : 1.f, a = std::fabs((*g[l])[i]);
+      for (int k = 0; k < in[l]; ++k) (*W[l])[(size_t)i * in[l] + k] *= s;
+      (*b[l])[i] *= s;
+      (*be[l])[i] /= a;
+      (*g[l])[i] = 1.f;
+      for (int n = 0; n < H; ++n) (*W[l + 1])[(size_t)n * in[l + 1] + i] *= a;
+    }
+  return true;
+}
+
+// Copies of one MLP's arrays, centred and folded for the fp32 model; the Layers are pointed at them.
+struct MlpCopy {
+  std::vector<std::vector<float>> W, b, g, be;
+  bool folded = false;
+};
+void prepare_mlp(Layer* lay, int L, int H, bool bf, bool fold, MlpCopy& c) {
+  if (bf) return;                                    // bf16 weights stay on the bf16 grid, as given
+  c.W.resize(L); c.b.resize(L); c.g.resize(L); c.be.resize(L);
+  std::vector<std::vector<float>*> W, b, g, be;
+  int in[4];
+  for (int l = 0; l < L; ++l) {
+    in[l] = lay[l].in;
+    centre_layer(lay[l].W, lay[l].b, H, lay[l].in, c.W[l], c.b[l]);
+    c.g[l].assign(lay[l].g, lay[l].g + H);
+    c.be[l].assign(lay[l].be, lay[l].be + H);
+    W.push_back(&c.W[l]); b.push_back(&c.b[l]); g.push_back(&c.g[l]); be.push_back(&c.be[l]);
+  }
+  c.folded = fold && fold_gamma(W, b, g, be, in, H);
+  for (int l = 0; l < L; ++l) lay[l] = {c.W[l].data(), c.b[l].data(), c.g[l].data(), c.be[l].data(), in[l]};
+}
+
+// A job's D starts from this bias.
+void set_bias(KernelPlan& pl, int job, const float* b) {
+  pl.biases.push_back(b);
+  pl.job_bias[job] = (int)pl.biases.size();
+}
+
+// The constant tiles a plan's biases are added with: D = ones * tile^T, one K step of 16.  Every row of
+// the ones tile [128, 16] is (1, 1, 1, 0, ...); row n of a bias tile [H, 16] is b[n] in three bf16 parts
+// (24 bits, all of an fp32 value), then zeros.  K-major without a swizzle: element (r, k) at byte
+// (r / 8) * 256 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2.
+std::vector<uint8_t> const_tiles(const KernelPlan& pl, int H) {
+  std::vector<uint8_t> t(128 * 32 + pl.biases.size() * H * 32, 0);
+  auto put = [](uint8_t* tile, int r, int k, uint16_t v) {
+    std::memcpy(tile + (r / 8) * 256 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2, &v, 2);
+  };
+  for (int r = 0; r < 128; ++r)
+    for (int k = 0; k < 3; ++k) put(t.data(), r, k, f32_to_bf16_rne(1.0f));
+  for (size_t i = 0; i < pl.biases.size(); ++i)
+    for (int n = 0; n < H; ++n) {
+      float v = pl.biases[i][n];
+      for (int k = 0; k < 3; ++k) {
+        const uint16_t part = f32_to_bf16_rne(v);
+        put(t.data() + 128 * 32 + i * H * 32, n, k, part);
+        v -= bf16_to_f32(part);
+      }
+    }
+  return t;
 }
 
 // Every whole H-float segment of a plan's vector block is one per-column vector (bias, gamma,
@@ -189,6 +294,20 @@ cudaError_t dev_alloc(void** p, size_t bytes) {
     return cudaErrorMemoryAllocation;
   }
   return cudaMalloc(p, bytes);
+}
+
+// A plan's vectors and constant tiles to the device.
+cudaError_t upload_plan(KernelPlan& pl, int H) {
+  const std::vector<uint8_t> tiles = const_tiles(pl, H);
+  pl.biases.clear();
+  const size_t vb = (pl.vecs.size() * 4 + 255) & ~size_t(255);
+  pl.const_bytes = (uint32_t)tiles.size();
+  cudaError_t err = dev_alloc((void**)&pl.d_vecs, vb + tiles.size());
+  if (err != cudaSuccess) { pl.d_vecs = nullptr; return err; }
+  pl.d_consts = (uint8_t*)pl.d_vecs + vb;
+  err = cudaMemcpy(pl.d_vecs, pl.vecs.data(), pl.vecs.size() * 4, cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = cudaMemcpy(pl.d_consts, tiles.data(), tiles.size(), cudaMemcpyHostToDevice);
+  return err;
 }
 
 // A kernel that waits, through the library's bounded wait, on an mbarrier nothing arrives on.
@@ -276,21 +395,33 @@ cudaError_t set_all_attrs() {
 template <TileKind K, int H, bool BF>
 cudaError_t launch_tile(gnn_ctx* c, const KernelPlan& pl, TileParams p, cudaStream_t st) {
   p.n_jobs = pl.n_jobs;
-  for (int j = 0; j < kMaxJobs; ++j) { p.job_mat[j] = pl.job_mat[j]; p.job_acc[j] = pl.job_acc[j]; }
+  // A lies in the region the previous job's D was written to, except where a job keeps its predecessor's
+  // regions: it accumulates into the same D, or (the P_d job, last of a node plan) reads the same A.
+  const bool node = K == TileKind::NodeEncoder || K == TileKind::NodeUpdate;
+  for (int j = 0, areg = 0; j < kMaxJobs; ++j) {
+    p.job_mat[j] = pl.job_mat[j];
+    p.job_acc[j] = pl.job_acc[j];
+    if (j > 0 && !(pl.job_acc[j] || (node && j == pl.n_jobs - 1))) areg ^= 1;
+    p.job_areg[j] = areg;
+    p.job_bias[j] = pl.job_bias[j];
+  }
+  p.folded = pl.folded ? 1 : 0;
+  p.consts = pl.d_consts;
+  p.const_bytes = pl.const_bytes;
   p.vecs = pl.d_vecs;
   p.n_vec_floats = (int)pl.vecs.size();
   p.wmats = pl.wmats ? pl.wmats : c->d_mats;
   p.mat_bytes = c->mat_bytes;
   p.n_tiles = (p.n_rows + kTileRows - 1) / kTileRows;
   if (p.n_tiles == 0) return cudaSuccess;
-  const uint32_t smem = tile_launch_smem<H, BF>(p.n_vec_floats);
+  const uint32_t smem = tile_launch_smem<H, BF>(p.n_vec_floats, p.const_bytes);
   const int grid = tile_grid(p.n_tiles, c->n_sm);
 #ifdef GNN_TRACE
   p.trace = ((int)K == c->trace_kind) ? c->trace : nullptr;
 #endif
   static const int group[7] = {1, 2, 3, 4, 5, 8, 9};   // NodeEncoder, EdgeEncoder, EdgeUpdate, NodeUpdate, Classifier, Filter, Embed
   const int pr = prof_begin(c, group[(int)K], 1, st);
-  const cudaError_t err = launch_pdl(mlp_tile_kernel<K, H, BF>, grid, kThreads, smem, st, p);
+  const cudaError_t err = launch_pdl(mlp_tile_kernel<K, H, BF>, grid, TileRoles<K>::THREADS, smem, st, p);
   prof_end(c, pr, st);
   return err;
 }
@@ -315,9 +446,9 @@ int run_network(gnn_ctx* c, const float* x, int N, int E, float* scores, cudaStr
 
   cudaError_t le = cudaSuccess;                        // first launch error
   auto chk = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
-  TileParams pn = p; pn.n_rows = N; pn.n_feat = c->cfg.n_node_feat;
+  TileParams pn = p; pn.n_rows = N; pn.n_feat = pn.n_in = c->cfg.n_node_feat;
   chk(launch_tile<TileKind::NodeEncoder, H, BF>(c, c->plan[T > 0 ? 0 : 1], pn, st));
-  TileParams pe = p; pe.n_rows = E; pe.n_feat = 2;
+  TileParams pe = p; pe.n_rows = E; pe.n_in = 2;
   chk(launch_tile<TileKind::EdgeEncoder, H, BF>(c, c->plan[2], pe, st));
   for (int t = 1; t <= T; ++t) {
     chk(launch_tile<TileKind::EdgeUpdate, H, BF>(c, c->plan[3], pe, st));
@@ -470,23 +601,14 @@ int gnn_create(const gnn_config* cfg, const void* weights_host, size_t weights_b
   // mean over the H outputs.  That subtraction is linear, so it is folded into
   // the layer: each weight column and the bias are centred over the output
   // rows (W' = (I - 11^T/H) W, b' = b - mean(b)).  The kernels then receive
-  // zero-mean pre-activations and compute only the variance.  Centred copies
-  // are kept in `centred` and the Layer pointers redirected to them.
+  // zero-mean pre-activations and compute only the variance.  The hidden layers'
+  // gammas go into the weights around them (fold_gamma).  Centred and folded
+  // copies are kept in `copies` and the Layer pointers redirected to them.
   // The bf16 model keeps its weights as given (bf16 values): centring would take them off the
   // bf16 grid, so its kernels subtract the LayerNorm mean themselves.
   const bool bf = cfg->precision == GNN_PRECISION_BF16;
-  std::vector<std::vector<float>> centred;
-  centred.reserve(2 * N_MLP * L);
-  for (int m = 0; m < N_MLP && !bf; ++m)
-    for (int l = 0; l < L; ++l) {
-      Layer& ly = lay[m][l];
-      std::vector<float> Wc, bc;
-      centre_layer(ly.W, ly.b, H, ly.in, Wc, bc);
-      centred.push_back(std::move(Wc));
-      ly.W = centred.back().data();
-      centred.push_back(std::move(bc));
-      ly.b = centred.back().data();
-    }
+  MlpCopy copies[N_MLP];
+  for (int m = 0; m < N_MLP; ++m) prepare_mlp(lay[m], L, H, bf, true, copies[m]);
 
   gnn_ctx* c = new (std::nothrow) gnn_ctx();
   if (!c) return GNN_ERR_OOM;
@@ -509,10 +631,14 @@ int gnn_create(const gnn_config* cfg, const void* weights_host, size_t weights_b
   int deep[N_MLP][4];
   for (int m = 0; m < N_MLP; ++m)
     for (int l = 1; l < L; ++l) deep[m][l] = add_mat(&lay[m][l], 0);
+  const int in_node = add_mat(&lay[NODE_ENC][0], -1), in_edge = add_mat(&lay[EDGE_ENC][0], -1);   // input matrices
   c->mat_bytes = (bf ? 1u : 2u) * H * H * 2u;
   std::vector<uint8_t> packed((size_t)c->mat_bytes * mats.size());
-  for (size_t i = 0; i < mats.size(); ++i)
-    pack_block(mats[i].first->W, mats[i].first->in, mats[i].second, H, !bf, packed.data() + i * c->mat_bytes);
+  for (size_t i = 0; i < mats.size(); ++i) {
+    uint8_t* out = packed.data() + i * c->mat_bytes;
+    if (mats[i].second < 0) pack_input(mats[i].first->W, mats[i].first->in, H, bf, out, c->mat_bytes);
+    else pack_block(mats[i].first->W, mats[i].first->in, mats[i].second, H, !bf, out);
+  }
 
   // kernel plans
   auto jobs = [](KernelPlan& pl, std::initializer_list<int> ids, int acc_mask = 0) {
@@ -520,54 +646,54 @@ int gnn_create(const gnn_config* cfg, const void* weights_host, size_t weights_b
     for (int id : ids) { pl.job_acc[pl.n_jobs] = (acc_mask >> pl.n_jobs) & 1; pl.job_mat[pl.n_jobs++] = id; }
   };
   auto add_deep = [&](KernelPlan& pl, int m) {
-    for (int l = 1; l < L; ++l) { pl.job_acc[pl.n_jobs] = 0; pl.job_mat[pl.n_jobs++] = deep[m][l]; }
+    pl.folded = copies[m].folded;
+    for (int l = 1; l < L; ++l) {
+      set_bias(pl, pl.n_jobs, lay[m][l].b);
+      pl.job_acc[pl.n_jobs] = 0;
+      pl.job_mat[pl.n_jobs++] = deep[m][l];
+    }
   };
-  auto bgb = [&](std::vector<float>& v, int m, int l0) {
-    for (int l = l0; l < L; ++l) { push(v, lay[m][l].b, H); push(v, lay[m][l].g, H); push(v, lay[m][l].be, H); }
+  auto gb = [&](std::vector<float>& v, int m) {
+    for (int l = 0; l < L; ++l) push_ln(v, lay[m][l], H);
   };
   for (int target = 0; target < 2; ++target) {           // node encoder -> edge net / classifier
     KernelPlan& pl = c->plan[target];
-    pl.n_jobs = 0;
+    jobs(pl, {in_node});
+    set_bias(pl, 0, lay[NODE_ENC][0].b);
     add_deep(pl, NODE_ENC);
     pl.job_mat[pl.n_jobs++] = target == 0 ? en_s : cl_s;
     pl.job_mat[pl.n_jobs++] = target == 0 ? en_d : cl_d;
-    for (int k = 0; k < Fn; ++k)                        // first-layer weight, transposed
-      for (int i = 0; i < H; ++i) pl.vecs.push_back(lay[NODE_ENC][0].W[(size_t)i * Fn + k]);
-    bgb(pl.vecs, NODE_ENC, 0);
-    push(pl.vecs, lay[target == 0 ? EDGE_NET : CLASSIFIER][0].b, H);
+    gb(pl.vecs, NODE_ENC);
+    set_bias(pl, pl.n_jobs - 1, lay[target == 0 ? EDGE_NET : CLASSIFIER][0].b);   // P_d carries it
   }
   {  // edge encoder
     KernelPlan& pl = c->plan[2];
-    pl.n_jobs = 0;
+    jobs(pl, {in_edge});
+    set_bias(pl, 0, lay[EDGE_ENC][0].b);
     add_deep(pl, EDGE_ENC);
-    for (int k = 0; k < 2; ++k)
-      for (int i = 0; i < H; ++i) pl.vecs.push_back(lay[EDGE_ENC][0].W[(size_t)i * 2 + k]);
-    bgb(pl.vecs, EDGE_ENC, 0);
+    gb(pl.vecs, EDGE_ENC);
   }
   {  // edge update
     KernelPlan& pl = c->plan[3];
     jobs(pl, {en_e});
     add_deep(pl, EDGE_NET);
-    push(pl.vecs, lay[EDGE_NET][0].g, H);
-    push(pl.vecs, lay[EDGE_NET][0].be, H);
-    bgb(pl.vecs, EDGE_NET, 1);
+    gb(pl.vecs, EDGE_NET);
   }
   for (int target = 0; target < 2; ++target) {           // node update -> edge net / classifier
     KernelPlan& pl = c->plan[4 + target];
     jobs(pl, {nn_h, nn_a}, 0b10);
+    set_bias(pl, 0, lay[NODE_NET][0].b);
     add_deep(pl, NODE_NET);
     pl.job_acc[pl.n_jobs] = 0; pl.job_mat[pl.n_jobs++] = target == 0 ? en_s : cl_s;
     pl.job_acc[pl.n_jobs] = 0; pl.job_mat[pl.n_jobs++] = target == 0 ? en_d : cl_d;
-    bgb(pl.vecs, NODE_NET, 0);
-    push(pl.vecs, lay[target == 0 ? EDGE_NET : CLASSIFIER][0].b, H);
+    gb(pl.vecs, NODE_NET);
+    set_bias(pl, pl.n_jobs - 1, lay[target == 0 ? EDGE_NET : CLASSIFIER][0].b);   // P_d carries it
   }
   {  // classifier
     KernelPlan& pl = c->plan[6];
     jobs(pl, {cl_e});
     add_deep(pl, CLASSIFIER);
-    push(pl.vecs, lay[CLASSIFIER][0].g, H);
-    push(pl.vecs, lay[CLASSIFIER][0].be, H);
-    bgb(pl.vecs, CLASSIFIER, 1);
+    gb(pl.vecs, CLASSIFIER);
     push(pl.vecs, head_w, H);
     push(pl.vecs, head_b, 1);
   }
@@ -575,11 +701,7 @@ int gnn_create(const gnn_config* cfg, const void* weights_host, size_t weights_b
   for (int i = 0; i < 7; ++i) finish_vecs(c->plan[i].vecs, H);
   err = dev_alloc((void**)&c->d_mats, packed.size());
   if (err == cudaSuccess) err = cudaMemcpy(c->d_mats, packed.data(), packed.size(), cudaMemcpyHostToDevice);
-  for (int i = 0; i < 7 && err == cudaSuccess; ++i) {
-    err = dev_alloc((void**)&c->plan[i].d_vecs, c->plan[i].vecs.size() * 4);
-    if (err == cudaSuccess)
-      err = cudaMemcpy(c->plan[i].d_vecs, c->plan[i].vecs.data(), c->plan[i].vecs.size() * 4, cudaMemcpyHostToDevice);
-  }
+  for (int i = 0; i < 7 && err == cudaSuccess; ++i) err = upload_plan(c->plan[i], H);
 #ifdef GNN_TRACE
   if (err == cudaSuccess) err = cudaMalloc(&c->trace, 3 * kTraceEvents * 8);
   if (err == cudaSuccess) err = cudaMemset(c->trace, 0, 3 * kTraceEvents * 8);
@@ -678,30 +800,28 @@ int gnn_filter_load(gnn_ctx* ctx, const void* weights_host, size_t weights_bytes
     f += (size_t)H * in + 3 * H;
   }
   const float* head = f;
-  std::vector<std::vector<float>> centred(2 * L);
-  if (!bf)
-    for (int l = 0; l < L; ++l) {
-      centre_layer(lay[l].W, lay[l].b, H, lay[l].in, centred[2 * l], centred[2 * l + 1]);
-      lay[l].W = centred[2 * l].data();
-      lay[l].b = centred[2 * l + 1].data();
-    }
+  MlpCopy copy;
+  prepare_mlp(lay.data(), L, H, bf, true, copy);
   KernelPlan pl;
-  for (int l = 1; l < L; ++l) { pl.job_acc[pl.n_jobs] = 0; pl.job_mat[pl.n_jobs] = l - 1; ++pl.n_jobs; }
-  for (int k = 0; k < 2 * Fn; ++k)                   // first-layer weight, transposed
-    for (int i = 0; i < H; ++i) pl.vecs.push_back(lay[0].W[(size_t)i * 2 * Fn + k]);
-  for (int l = 0; l < L; ++l) { push(pl.vecs, lay[l].b, H); push(pl.vecs, lay[l].g, H); push(pl.vecs, lay[l].be, H); }
+  pl.folded = copy.folded;
+  for (int l = 0; l < L; ++l) {                       // job and matrix l: layer l, the first an input matrix
+    set_bias(pl, l, lay[l].b);
+    pl.job_mat[l] = l;
+  }
+  pl.n_jobs = L;
+  for (int l = 0; l < L; ++l) push_ln(pl.vecs, lay[l], H);
   push(pl.vecs, head, H + 1);
   finish_vecs(pl.vecs, H);
-  std::vector<uint8_t> packed((size_t)ctx->mat_bytes * (L - 1));
-  for (int l = 1; l < L; ++l) pack_block(lay[l].W, H, 0, H, !bf, packed.data() + (size_t)(l - 1) * ctx->mat_bytes);
+  std::vector<uint8_t> packed((size_t)ctx->mat_bytes * L);
+  pack_input(lay[0].W, lay[0].in, H, bf, packed.data(), ctx->mat_bytes);
+  for (int l = 1; l < L; ++l) pack_block(lay[l].W, H, 0, H, !bf, packed.data() + (size_t)l * ctx->mat_bytes);
   // replace a previous filter
   if (ctx->filter_plan.d_vecs) { cudaFree(ctx->filter_plan.d_vecs); ctx->filter_plan.d_vecs = nullptr; }
   if (ctx->d_filter_mats) { cudaFree(ctx->d_filter_mats); ctx->d_filter_mats = nullptr; }
   ctx->filter_layers = 0;
   cudaError_t err = dev_alloc((void**)&ctx->d_filter_mats, packed.size());
   if (err == cudaSuccess) err = cudaMemcpy(ctx->d_filter_mats, packed.data(), packed.size(), cudaMemcpyHostToDevice);
-  if (err == cudaSuccess) err = dev_alloc((void**)&pl.d_vecs, pl.vecs.size() * 4);
-  if (err == cudaSuccess) err = cudaMemcpy(pl.d_vecs, pl.vecs.data(), pl.vecs.size() * 4, cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = upload_plan(pl, H);
   if (err != cudaSuccess) {
     if (pl.d_vecs) cudaFree(pl.d_vecs);
     if (ctx->d_filter_mats) { cudaFree(ctx->d_filter_mats); ctx->d_filter_mats = nullptr; }
@@ -733,6 +853,7 @@ int gnn_filter_edges(gnn_ctx* ctx, const float* node_feats, const int32_t* edge_
   p.n_nodes = N;
   p.n_layers = ctx->filter_layers;
   p.n_feat = ctx->cfg.n_node_feat;
+  p.n_in = 2 * p.n_feat;
   p.eps = ctx->filter_eps;
   p.x = node_feats;
   p.x_stride = ctx->cfg.n_node_feat;
@@ -783,29 +904,27 @@ int gnn_embed_load(gnn_ctx* ctx, const void* weights_host, size_t weights_bytes)
     f += (size_t)H * in + 3 * H;
   }
   const float* wout = f;                                  // [D, H] then b_out [D]
-  std::vector<std::vector<float>> centred(2 * L);
-  if (!bf)
-    for (int l = 0; l < L; ++l) {
-      centre_layer(lay[l].W, lay[l].b, H, lay[l].in, centred[2 * l], centred[2 * l + 1]);
-      lay[l].W = centred[2 * l].data();
-      lay[l].b = centred[2 * l + 1].data();
-    }
+  MlpCopy copy;
+  prepare_mlp(lay.data(), L, H, bf, false, copy);
   KernelPlan pl;
-  for (int l = 1; l < L; ++l) { pl.job_acc[pl.n_jobs] = 0; pl.job_mat[pl.n_jobs] = l - 1; ++pl.n_jobs; }
-  for (int k = 0; k < Fn; ++k)                        // first-layer weight, transposed
-    for (int i = 0; i < H; ++i) pl.vecs.push_back(lay[0].W[(size_t)i * Fn + k]);
-  for (int l = 0; l < L; ++l) { push(pl.vecs, lay[l].b, H); push(pl.vecs, lay[l].g, H); push(pl.vecs, lay[l].be, H); }
+  pl.folded = copy.folded;
+  for (int l = 0; l < L; ++l) {                       // job and matrix l: layer l, the first an input matrix
+    set_bias(pl, l, lay[l].b);
+    pl.job_mat[l] = l;
+  }
+  pl.n_jobs = L;
+  for (int l = 0; l < L; ++l) push_ln(pl.vecs, lay[l], H);
   push(pl.vecs, wout, (size_t)D * H + D);
   finish_vecs(pl.vecs, H);
-  std::vector<uint8_t> packed((size_t)ctx->mat_bytes * (L - 1));
-  for (int l = 1; l < L; ++l) pack_block(lay[l].W, H, 0, H, !bf, packed.data() + (size_t)(l - 1) * ctx->mat_bytes);
+  std::vector<uint8_t> packed((size_t)ctx->mat_bytes * L);
+  pack_input(lay[0].W, lay[0].in, H, bf, packed.data(), ctx->mat_bytes);
+  for (int l = 1; l < L; ++l) pack_block(lay[l].W, H, 0, H, !bf, packed.data() + (size_t)l * ctx->mat_bytes);
   if (ctx->embed_plan.d_vecs) { cudaFree(ctx->embed_plan.d_vecs); ctx->embed_plan.d_vecs = nullptr; }
   if (ctx->d_embed_mats) { cudaFree(ctx->d_embed_mats); ctx->d_embed_mats = nullptr; }
   ctx->embed_layers = 0;
   cudaError_t err = dev_alloc((void**)&ctx->d_embed_mats, packed.size());
   if (err == cudaSuccess) err = cudaMemcpy(ctx->d_embed_mats, packed.data(), packed.size(), cudaMemcpyHostToDevice);
-  if (err == cudaSuccess) err = dev_alloc((void**)&pl.d_vecs, pl.vecs.size() * 4);
-  if (err == cudaSuccess) err = cudaMemcpy(pl.d_vecs, pl.vecs.data(), pl.vecs.size() * 4, cudaMemcpyHostToDevice);
+  if (err == cudaSuccess) err = upload_plan(pl, H);
   if (err != cudaSuccess) {
     if (pl.d_vecs) cudaFree(pl.d_vecs);
     if (ctx->d_embed_mats) { cudaFree(ctx->d_embed_mats); ctx->d_embed_mats = nullptr; }
@@ -827,7 +946,7 @@ int gnn_embed(gnn_ctx* ctx, const float* node_feats, int64_t n_nodes, float* emb
   p.n_rows = (int)n_nodes;
   p.n_nodes = (int)n_nodes;
   p.n_layers = ctx->embed_layers;
-  p.n_feat = ctx->cfg.n_node_feat;
+  p.n_feat = p.n_in = ctx->cfg.n_node_feat;
   p.eps = ctx->embed_eps;
   p.x = node_feats;
   p.x_stride = ctx->cfg.n_node_feat;

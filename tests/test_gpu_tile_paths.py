@@ -1,0 +1,75 @@
+"""Branches of the tile kernels' launch plans, at the sizes where they turn (through the C ABI):
+
+* gammas folded into the weights (negative ones among them) and gammas that cannot be folded (zero, tiny);
+* tile counts around one per CTA and one per worker group, resident and streamed weights (L = 4), with
+  ragged last tiles and groups without a tile in the last round;
+* first-layer inputs of one and two K steps, the narrowest and the widest."""
+import numpy as np
+import pytest
+
+from oracle import gnn_oracle as O
+from paper_2402_09633_gb300 import synthetic as S
+from tests.gpu_util import check_parity, logits_from_scores, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+def _gammas(W, how, rng):
+    out = dict(W)
+    for m in S.MLP_NAMES:
+        layers = []
+        for (w, b, g, be) in W[m]:
+            g = g.copy()
+            if how == "negative":
+                g *= np.where(rng.random(g.size) < 0.4, -1.0, 1.0).astype(np.float32)
+            elif how == "zero":                      # the layer's output there is relu(beta)
+                g[:: 7] = 0.0
+                g[3] = 1e-20
+            layers.append((w, b, g, be))
+        out[m] = layers
+    return out
+
+
+@pytest.mark.parametrize("how", ["negative", "zero"])
+@pytest.mark.parametrize("H,L", [(128, 3), (64, 2)])
+def test_gammas_folded_and_not(how, H, L):
+    cfg = S.ModelConfig(5, 2, H, 2, L)
+    W = _gammas(S.init_weights(cfg, 4), how, np.random.default_rng(H + L))
+    x, ei = S.random_graph(900, 3000, 5, seed=L)
+    s, rc = run_gpu(cfg, W, x, ei)
+    assert rc == 0
+    check_parity(s, W, x, ei, cfg.n_iters)
+
+
+# 152 CTAs on a GB300: one tile or one round per CTA, one tile more, a last round with one group only
+@pytest.mark.parametrize("tiles,last", [(1, 1), (152, 128), (153, 1), (3 * 152, 127), (3 * 152 + 1, 1), (5 * 152, 64)])
+@pytest.mark.parametrize("L", [3, 4])
+def test_tile_counts(tiles, last, L):
+    cfg = S.ModelConfig(3, 2, 128, 1, L)
+    W = S.init_weights(cfg, 6)
+    n_edges = (tiles - 1) * 128 + last
+    x, ei = S.random_graph(max(n_edges // 2, 2), n_edges, 3, seed=tiles)
+    s, rc = run_gpu(cfg, W, x, ei)
+    assert rc == 0
+    check_parity(s, W, x, ei, cfg.n_iters)
+
+
+@pytest.mark.parametrize("feat", [2, 8, 9, 16])
+@pytest.mark.parametrize("H,L", [(128, 4), (64, 2)])
+def test_input_widths_of_encoder_and_filter(feat, H, L):
+    import torch
+    from paper_2402_09633_gb300 import InteractionNetwork
+    cfg = S.ModelConfig(feat, 2, H, 1, L)
+    W, fw = S.init_weights(cfg, 1), S.init_filter_weights(cfg, 2)
+    x, ei = S.random_graph(700, 2100, feat, seed=feat)
+    x = x * np.float32(3.0)                          # beyond the unit range the features usually have
+    x[:, 1] = np.clip(x[:, 1] / 3, -1, 1)
+    net = InteractionNetwork(cfg, S.pack_blob(cfg, W))
+    net.load_filter(S.pack_filter_blob(cfg, fw))
+    xs, es = torch.from_numpy(x).cuda(), torch.from_numpy(ei).cuda()
+    check_parity(net.infer(xs, es).cpu().numpy(), W, x, ei, 1)
+    sc, _, _ = net.filter_edges(xs, es, 0.5)
+    _, want = O.filter_scores(fw, x, ei, cfg.ln_eps, return_logits=True)
+    assert np.abs(logits_from_scores(sc.cpu().numpy()) - want).max() <= 2e-3
+    assert net.status() == 0
+    net.close()
