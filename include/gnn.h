@@ -169,7 +169,7 @@ int gnn_infer_host(gnn_ctx* ctx, const float* node_feats, const int32_t* edge_in
  * for that many.  The order
  * of the edges is deterministic.  Uses a scratch buffer of the context (grown on demand,
  * synchronous then): besides the sorted copies, 128 bytes per hit for the partner chains the
- * counting pass keeps (see gnn_debug_graph_pool).  Errors: INVALID_ARG (radius <= 0, emb_dim out
+ * counting pass keeps (see gnn_debug_graph_pool) and 64 (128 for emb_dim > 8) for the pair filter.  Errors: INVALID_ARG (radius <= 0, emb_dim out
  * of range, null pointer, bad sizes), OOM, CUDA.
  */
 int gnn_embed_load(gnn_ctx* ctx, const void* weights_host, size_t weights_bytes);

@@ -994,7 +994,10 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   // buffers each), per-hit counts, per-block sums, radix histograms, cell starts, the pool counter
   const int nb = (int)blocks_for(N, tb);
   const size_t chain_ints = ((size_t)N + (size_t)pool) * kFrnnChunk;
-  const size_t need = 4 * (size_t)chunks * N + chain_ints + 6 * (size_t)N + (size_t)nb + 256 * (size_t)tiles +
+  // B fragments of the pair filter: 16 bytes x 32 lanes per eight hits and set of eight coordinates
+  const int sets = (chunks + 1) / 2;
+  const size_t frag_ints = ((size_t)N + 7) / 8 * 128 * (size_t)sets;
+  const size_t need = 4 * (size_t)chunks * N + frag_ints + chain_ints + 6 * (size_t)N + (size_t)nb + 256 * (size_t)tiles +
                       (size_t)n_cells + 2;
   if (need > ctx->aux_ints) {
     if (ctx->aux) { cudaStreamSynchronize(st); cudaFree(ctx->aux); ctx->aux = nullptr; ctx->aux_ints = 0; }
@@ -1003,7 +1006,8 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
     ctx->aux_ints = need;
   }
   float4* emb_s = (float4*)ctx->aux;
-  int* chains = (int*)(ctx->aux + 4 * (size_t)chunks * N);
+  uint4* frag = (uint4*)(ctx->aux + 4 * (size_t)chunks * N);
+  int* chains = (int*)frag + frag_ints;
   float* r_s = (float*)(chains + chain_ints);
   int* keys_a = (int*)(r_s + N);
   int* keys_b = keys_a + N;
@@ -1035,18 +1039,20 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   const float r2 = radius * radius;
   const int xs = ctx->cfg.n_node_feat;
   const int sb = (int)blocks_for(N, kScanBlock);
-  const int pb = (int)blocks_for(N, kFrnnPairsThreads);
+  const int pb = (int)blocks_for(N, kFrnnBlockQueries);
+  const int fb = (int)blocks_for(blocks_for(N, 8) * (int64_t)32, tb);
   switch (chunks * 8 + K) {
 #define GNN_FRNN_CASE(CH, KK)                                                                                    \
   case CH * 8 + KK:                                                                                              \
     frnn_gather_kernel<CH><<<nb, tb, 0, st>>>(embedding, node_feats, xs, N, emb_dim, vin, emb_s, r_s);         \
-    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, r_s, N, r2, grid, kin, vin, cell_start, \
+    frnn_fragments_kernel<CH><<<fb, tb, 0, st>>>(emb_s, N, frag);                                                \
+    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, frag, r_s, N, r2, grid, kin, vin, cell_start, \
                                                                 0, counts, nullptr, 0, nullptr, chains,          \
                                                                 next_chunk, pool, ctx->d_err);                   \
     scan_reduce_kernel<<<sb, kScanBlock, 0, st>>>(counts, N, block_sums);                                      \
     compact_scan_kernel<<<1, 1024, 0, st>>>(block_sums, sb, n_edges);                                            \
     scan_apply_kernel<<<sb, kScanBlock, 0, st>>>(counts, N, block_sums);                                       \
-    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, r_s, N, r2, grid, kin, vin, cell_start, \
+    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, frag, r_s, N, r2, grid, kin, vin, cell_start, \
                                                                 1, counts, n_edges, (int)max_edges, edge_index,  \
                                                                 chains, next_chunk, pool, ctx->d_err);           \
     frnn_copy_kernel<<<nb, tb, 0, st>>>(r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index);      \
