@@ -57,8 +57,7 @@ __device__ __forceinline__ int frnn_coord(float e, int grid) {
 // Cell key of every hit: its cell over the first K coordinates (missing ones count as cell 0),
 // row-major with the last gridded coordinate fastest.
 template <int K>
-__global__ void frnn_cell_kernel(const float* __restrict__ emb, int n, int dim, int grid, int* __restrict__ keys,
-                                 int* __restrict__ vals) {
+__global__ void frnn_cell_kernel(const float* __restrict__ emb, int n, int dim, int grid, int* __restrict__ keys) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float* e = emb + (size_t)i * dim;
@@ -66,7 +65,6 @@ __global__ void frnn_cell_kernel(const float* __restrict__ emb, int n, int dim, 
 #pragma unroll
   for (int k = 0; k < K; ++k) key = key * grid + (k < dim ? frnn_coord(e[k], grid) : 0);
   keys[i] = key;
-  vals[i] = i;
 }
 
 // Sorted copies: emb_s [n, 4 * CH] (zero-padded), r_s [n] = x[ids[t], 0].

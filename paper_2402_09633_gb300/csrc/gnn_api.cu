@@ -86,7 +86,7 @@ struct gnn_ctx {
   // workspace
   void* ws = nullptr;
   int64_t cap_nodes = -1, cap_edges = -1;
-  int *keys_a = nullptr, *keys_b = nullptr, *vals_a = nullptr, *vals_b = nullptr, *src_c = nullptr;
+  int *keys_a = nullptr, *keys_b = nullptr, *vals_a = nullptr, *vals_b = nullptr;
   int *hist = nullptr, *perm = nullptr, *src_sorted = nullptr, *dst_sorted = nullptr, *rowptr = nullptr;
   int* key_sorted = nullptr;
   void *e = nullptr, *h = nullptr, *agg = nullptr;  // stored states (fp32 or bf16 per precision)
@@ -478,14 +478,14 @@ int ensure_workspace(gnn_ctx* c, int64_t N, int64_t E) {
   const int64_t n = N > c->cap_nodes ? N : c->cap_nodes;
   const int64_t e = E > c->cap_edges ? E : c->cap_edges;
   const int64_t H = c->cfg.hidden;
-  const int64_t rs_tiles = (e + kRadixTile - 1) / kRadixTile;
+  const int64_t hist_bytes = 4 * (int64_t)radix_hist_ints((size_t)e);
   auto al = [](int64_t b) { return (b + 255) & ~int64_t(255); };
   const int64_t sz_e_int = al(4 * (e > 0 ? e : 1));
   // edge and node state use the row-tiled layout: rows padded to whole 128-row tiles
   const int64_t e_pad = (e + kTileRows - 1) / kTileRows * kTileRows;
   const int64_t n_pad = (n + kTileRows - 1) / kTileRows * kTileRows;
   const int64_t se = state_bytes(c);                   // stored-state element: fp32 or bf16
-  const int64_t total = 8 * sz_e_int + al(4 * 256 * (rs_tiles > 0 ? rs_tiles : 1)) + al(4 * (n + 1)) +
+  const int64_t total = 7 * sz_e_int + al(hist_bytes) + al(4 * (n + 1)) +
                         al(se * e_pad * H) + 2 * al(se * n_pad * H) + 2 * al(4 * n * H);
   free_workspace(c);
   void* ws = nullptr;
@@ -496,9 +496,9 @@ int ensure_workspace(gnn_ctx* c, int64_t N, int64_t E) {
   auto take = [&](int64_t bytes) { uint8_t* r = q; q += al(bytes); return r; };
   c->keys_a = (int*)take(4 * e); c->keys_b = (int*)take(4 * e);
   c->vals_a = (int*)take(4 * e); c->vals_b = (int*)take(4 * e);
-  c->src_c = (int*)take(4 * e); c->perm = (int*)take(4 * e);
+  c->perm = (int*)take(4 * e);
   c->src_sorted = (int*)take(4 * e); c->dst_sorted = (int*)take(4 * e);
-  c->hist = (int*)take(4 * 256 * (rs_tiles > 0 ? rs_tiles : 1));
+  c->hist = (int*)take(hist_bytes);
   c->rowptr = (int*)take(4 * (n + 1));
   c->e = take(se * e_pad * H);
   c->h = take(se * n_pad * H);
@@ -510,34 +510,52 @@ int ensure_workspace(gnn_ctx* c, int64_t N, int64_t E) {
   return GNN_OK;
 }
 
-int build_csr(gnn_ctx* c, const int32_t* ei, int N, int E, cudaStream_t st) {
-  const int tb = 256;
-  int n_bits = 0;
-  while (n_bits < 31 && (N >> n_bits) != 0) ++n_bits;
-  const int n_passes = ((n_bits > 0 ? n_bits : 1) + 7) / 8;
-  const int pr = prof_begin(c, 0, 3 + 3 * n_passes, st);
-  cudaError_t le = cudaSuccess;                        // first launch error
-  auto chk = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
-  chk(launch_pdl(csr_keys_kernel, blocks_for(E, tb), tb, 0, st, ei, E, N, c->keys_a, c->vals_a, c->src_c, c->d_err));
-  int bits = 0;
-  while (bits < 31 && (N >> bits) != 0) ++bits;        // keys lie in [0, N]
-  if (bits == 0) bits = 1;
-  const int passes = (bits + 7) / 8;
-  const int tiles = (int)blocks_for(E, kRadixTile);
-  int *kin = c->keys_a, *vin = c->vals_a, *kout = c->keys_b, *vout = c->vals_b;
-  for (int ps = 0; ps < passes; ++ps) {
-    const int shift = 8 * ps;
-    chk(launch_pdl(radix_count_kernel, tiles, kRadixThreads, 0, st, (const int*)kin, E, shift, tiles, c->hist));
-    chk(launch_pdl(radix_offsets_kernel, 1, kOffsetsThreads, 0, st, c->hist, tiles));
-    chk(launch_pdl(radix_scatter_kernel, tiles, kRadixThreads, 0, st, (const int*)kin, (const int*)vin, kout, vout, E,
-                   shift, tiles, (const int*)c->hist));
-    int* t = kin; kin = kout; kout = t;
-    t = vin; vin = vout; vout = t;
+// Stable sort of n keys in [0, max_key] read through `src` (first pass), values = positions in it, by
+// passes that write keys_out[0], keys_out[1], ... in turn (two buffers each).  Returns the index of the
+// buffers that hold the result.
+template <typename Src>
+int launch_radix_sort(const Src& src, int n, int max_key, int* const* keys, int* const* vals, int* hist, cudaStream_t st,
+                      cudaError_t* err) {
+  auto chk = [&](cudaError_t e) { if (*err == cudaSuccess) *err = e; };
+  const RadixPlan plan = radix_plan(max_key);
+  const int tiles = (int)blocks_for(n, kRadixTile), bins = 1 << plan.digit;
+  int* totals = hist + (size_t)tiles * bins;
+  for (int ps = 0; ps < plan.passes; ++ps) {
+    const int shift = plan.digit * ps, out = ps & 1;
+    const RadixPairs pairs{keys[out ^ 1], vals[out ^ 1]};
+    if (ps == 0) chk(launch_pdl(radix_count_kernel<Src>, tiles, kRadixThreads, 0, st, src, n, shift, bins, tiles, hist));
+    else chk(launch_pdl(radix_count_kernel<RadixPairs>, tiles, kRadixThreads, 0, st, pairs, n, shift, bins, tiles, hist));
+    chk(launch_pdl(radix_scan_kernel, blocks_for(bins, kRadixWarps), kRadixThreads, 0, st, hist, bins, tiles, totals));
+    if (ps == 0)
+      chk(launch_pdl(radix_scatter_kernel<Src>, tiles, kRadixThreads, 0, st, src, keys[out], vals[out], n, shift, bins,
+                     tiles, (const int*)hist, (const int*)totals));
+    else
+      chk(launch_pdl(radix_scatter_kernel<RadixPairs>, tiles, kRadixThreads, 0, st, pairs, keys[out], vals[out], n, shift,
+                     bins, tiles, (const int*)hist, (const int*)totals));
   }
-  c->key_sorted = kin;
-  chk(launch_pdl(csr_gather_kernel, blocks_for(E, tb), tb, 0, st, (const int*)kin, (const int*)vin,
-                 (const int*)c->src_c, E, N, c->perm, c->src_sorted, c->dst_sorted));
-  chk(launch_pdl(csr_rowptr_kernel, blocks_for((int64_t)N + 1, tb), tb, 0, st, (const int*)kin, E, N, c->rowptr));
+  return (plan.passes - 1) & 1;
+}
+
+// The destination-keyed CSR of ei [2, E] into perm, src_sorted, dst_sorted (may be null) and rowptr;
+// returns the sorted keys through key_sorted.
+cudaError_t launch_csr(const int32_t* ei, int N, int E, int* const* keys, int* const* vals, int* hist, int* perm,
+                       int* src_sorted, int* dst_sorted, int* rowptr, uint32_t* d_err, int** key_sorted, cudaStream_t st) {
+  constexpr int tb = 256;
+  cudaError_t err = cudaSuccess;                       // first launch error
+  const int k = launch_radix_sort(RadixEdges{ei, E, N, d_err}, E, N, keys, vals, hist, st, &err);
+  const int64_t threads = E > (int64_t)N + 1 ? E : (int64_t)N + 1;
+  const cudaError_t e = launch_pdl(csr_finish_kernel, blocks_for(threads, tb), tb, 0, st, ei, (const int*)keys[k],
+                                   (const int*)vals[k], E, N, perm, src_sorted, dst_sorted, rowptr);
+  if (key_sorted) *key_sorted = keys[k];
+  return err != cudaSuccess ? err : e;
+}
+
+int build_csr(gnn_ctx* c, const int32_t* ei, int N, int E, cudaStream_t st) {
+  const int pr = prof_begin(c, 0, 3 * radix_plan(N).passes + 1, st);
+  int* const keys[2] = {c->keys_a, c->keys_b};
+  int* const vals[2] = {c->vals_a, c->vals_b};
+  const cudaError_t le = launch_csr(ei, N, E, keys, vals, c->hist, c->perm, c->src_sorted, c->dst_sorted, c->rowptr,
+                                    c->d_err, &c->key_sorted, st);
   prof_end(c, pr, st);
   const cudaError_t err = le != cudaSuccess ? le : cudaGetLastError();
   return err == cudaSuccess ? GNN_OK : cuda_fail(err);
@@ -984,7 +1002,6 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   const int grid = frnn_grid(radius, K);
   int n_cells = 1;
   for (int k = 0; k < K; ++k) n_cells *= grid;
-  const int tiles = (int)blocks_for(N, kRadixTile);
   const int chunks = (emb_dim + 3) / 4;                   // float4 chunks per sorted embedding
   // partner chains kept by the counting pass: one first chunk per hit, pool chunks after them (a hit
   // whose chain cannot grow is searched again by the writing pass)
@@ -997,7 +1014,7 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   // B fragments of the pair filter: 16 bytes x 32 lanes per eight hits and set of eight coordinates
   const int sets = (chunks + 1) / 2;
   const size_t frag_ints = ((size_t)N + 7) / 8 * 128 * (size_t)sets;
-  const size_t need = 4 * (size_t)chunks * N + frag_ints + chain_ints + 6 * (size_t)N + (size_t)nb + 256 * (size_t)tiles +
+  const size_t need = 4 * (size_t)chunks * N + frag_ints + chain_ints + 6 * (size_t)N + (size_t)nb + radix_hist_ints(N) +
                       (size_t)n_cells + 2;
   if (need > ctx->aux_ints) {
     if (ctx->aux) { cudaStreamSynchronize(st); cudaFree(ctx->aux); ctx->aux = nullptr; ctx->aux_ints = 0; }
@@ -1014,23 +1031,19 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   int* vals_a = keys_b + N;
   int* vals_b = vals_a + N;
   int* counts = vals_b + N;
+  int* cells = counts;                                    // the hits' cells, until they are sorted
   int* block_sums = counts + N;
   int* hist = block_sums + nb;
-  int* cell_start = hist + 256 * (size_t)tiles;
+  int* cell_start = hist + radix_hist_ints(N);
   int* next_chunk = cell_start + n_cells + 1;
-  if (K == 4) frnn_cell_kernel<4><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, keys_a, vals_a);
-  else frnn_cell_kernel<3><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, keys_a, vals_a);
-  int bits = 0;
-  while (bits < 31 && ((n_cells - 1) >> bits) != 0) ++bits;
-  const int passes = ((bits > 0 ? bits : 1) + 7) / 8;
-  int *kin = keys_a, *vin = vals_a, *kout = keys_b, *vout = vals_b;
-  for (int ps = 0; ps < passes; ++ps) {
-    radix_count_kernel<<<tiles, kRadixThreads, 0, st>>>(kin, N, 8 * ps, tiles, hist);
-    radix_offsets_kernel<<<1, kOffsetsThreads, 0, st>>>(hist, tiles);
-    radix_scatter_kernel<<<tiles, kRadixThreads, 0, st>>>(kin, vin, kout, vout, N, 8 * ps, tiles, hist);
-    int* t = kin; kin = kout; kout = t;
-    t = vin; vin = vout; vout = t;
-  }
+  if (K == 4) frnn_cell_kernel<4><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, cells);
+  else frnn_cell_kernel<3><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, cells);
+  int* const skeys[2] = {keys_a, keys_b};
+  int* const svals[2] = {vals_a, vals_b};
+  cudaError_t serr = cudaSuccess;
+  const int sorted = launch_radix_sort(RadixKeys{cells}, N, n_cells - 1, skeys, svals, hist, st, &serr);
+  if (serr != cudaSuccess) return cuda_fail(serr);
+  const int *kin = skeys[sorted], *vin = svals[sorted];
   csr_rowptr_kernel<<<blocks_for((int64_t)n_cells + 1, tb), tb, 0, st>>>(kin, N, n_cells, cell_start);
   {
     const cudaError_t e0 = cudaMemsetAsync(next_chunk, 0, sizeof(int), st);
@@ -1196,13 +1209,16 @@ int gnn_debug_copy(gnn_ctx* ctx, int which, void* dst, size_t bytes, gnn_stream_
 // ---------------------------------------------------------------------------
 // Allocation-free CSR build: the radix-sort scratch lives in one file-scope
 // device array instead of context workspace.  Layout (int32 words):
-// keys_a | keys_b | vals_a | vals_b | src_clamped (GNN_CSR_NOALLOC_MAX_EDGES
-// each) | per-tile digit histograms (256 x 256).  Host code must not use the
+// keys_a | keys_b | vals_a | vals_b (GNN_CSR_NOALLOC_MAX_EDGES each) | per-tile
+// digit counts and digit totals.  Host code must not use the
 // array's name as a device address: every call asks cudaGetSymbolAddress for
 // it, with the caller's device current.  The address is not cached, because it
 // belongs to the current context's copy of the module: it changes after
 // cudaDeviceReset and differs under another context on the same device.
-static_assert((GNN_CSR_NOALLOC_MAX_EDGES + kRadixTile - 1) / kRadixTile <= 256, "histogram area too small");
+static_assert(4ull * GNN_CSR_NOALLOC_MAX_EDGES +
+                      ((GNN_CSR_NOALLOC_MAX_EDGES + kRadixTile - 1) / kRadixTile + 1) * (unsigned long long)kRadixMaxBins <=
+                  GNN_CSR_NOALLOC_SCRATCH_BYTES / 4,
+              "count area too small");
 static __device__ __align__(256) unsigned char g_csr_noalloc_scratch[GNN_CSR_NOALLOC_SCRATCH_BYTES];
 
 extern "C" int gnn_csr_build_noalloc(const int32_t* edge_index, int64_t n_nodes, int64_t n_edges,
@@ -1223,30 +1239,11 @@ extern "C" int gnn_csr_build_noalloc(const int32_t* edge_index, int64_t n_nodes,
     return ce == cudaSuccess ? GNN_OK : cuda_fail(ce);
   }
   int* words = reinterpret_cast<int*>(scratch);
-  int* keys_a = words;
-  int* keys_b = keys_a + GNN_CSR_NOALLOC_MAX_EDGES;
-  int* vals_a = keys_b + GNN_CSR_NOALLOC_MAX_EDGES;
-  int* vals_b = vals_a + GNN_CSR_NOALLOC_MAX_EDGES;
-  int* src_c = vals_b + GNN_CSR_NOALLOC_MAX_EDGES;
-  int* hist = src_c + GNN_CSR_NOALLOC_MAX_EDGES;
-  csr_keys_kernel<<<blocks_for(E, tb), tb, 0, st>>>(edge_index, E, N, keys_a, vals_a, src_c, nullptr);
-  int bits = 0;
-  while (bits < 31 && (N >> bits) != 0) ++bits;   // keys lie in [0, N]
-  if (bits == 0) bits = 1;
-  const int passes = (bits + 7) / 8;
-  const int tiles = (int)blocks_for(E, kRadixTile);
-  int *kin = keys_a, *vin = vals_a, *kout = keys_b, *vout = vals_b;
-  for (int ps = 0; ps < passes; ++ps) {
-    const int shift = 8 * ps;
-    radix_count_kernel<<<tiles, kRadixThreads, 0, st>>>(kin, E, shift, tiles, hist);
-    radix_offsets_kernel<<<1, kOffsetsThreads, 0, st>>>(hist, tiles);
-    radix_scatter_kernel<<<tiles, kRadixThreads, 0, st>>>(kin, vin, kout, vout, E, shift, tiles, hist);
-    int* t = kin; kin = kout; kout = t;
-    t = vin; vin = vout; vout = t;
-  }
-  // sorted keys in kin; kout is free and receives the (unused) clamped destinations
-  csr_gather_kernel<<<blocks_for(E, tb), tb, 0, st>>>(kin, vin, src_c, E, N, perm, src_sorted, kout);
-  csr_rowptr_kernel<<<blocks_for((int64_t)N + 1, tb), tb, 0, st>>>(kin, E, N, rowptr);
+  int* const keys[2] = {words, words + GNN_CSR_NOALLOC_MAX_EDGES};
+  int* const vals[2] = {words + 2 * GNN_CSR_NOALLOC_MAX_EDGES, words + 3 * GNN_CSR_NOALLOC_MAX_EDGES};
+  int* hist = words + 4 * GNN_CSR_NOALLOC_MAX_EDGES;
+  ce = launch_csr(edge_index, N, E, keys, vals, hist, perm, src_sorted, nullptr, rowptr, nullptr, nullptr, st);
+  if (ce != cudaSuccess) return cuda_fail(ce);
   ce = cudaGetLastError();
   return ce == cudaSuccess ? GNN_OK : cuda_fail(ce);
 }
