@@ -87,14 +87,17 @@ __global__ void frnn_gather_kernel(const float* __restrict__ emb, const float* _
 }
 
 // The tensor-core filter of the pair search.  With a = ah + al and b = bh + bl (bf16 parts) and the
-// squared norms in three bf16 parts each, one product of K = 32 (dimensions 0-7; 16 more for each of two
-// further sets of eight) gives
+// squared norms in three bf16 parts each, one product of K = 32 (dimensions 0-7; 32 more for eight
+// further ones) gives
 //   f = (1 - c)(|a|^2 + |b|^2) - 2 (ah bh + ah bl + al bh) - r2',  c = 2^-14, r2' slightly above r2.
 // Against the squared distance d the parts left out, the splits' rounding and the accumulation are off
 // by less than 3e-5 (|a|^2 + |b|^2) / 2 + 1e-5 (|a|^2 + |b|^2), under half of c (|a|^2 + |b|^2): a pair
-// with d < r2 never gives f >= 0.  Pairs with !(f >= 0) (NaN from infinities among them) are tested
-// exactly.  K slots: 0-7 -2ah.bh, 8-15 -2ah.bl, 16-23 -2al.bh, 24-26 |a|^2 parts x 1, 27-29 1 x |b|^2 parts.
+// with d < r2 never gives f >= 0.  Only pairs with f < 0 are tested exactly.  A hit that is not finite
+// or whose squared norm passes 1e18 is "wild": its operands are zero and its norm slot -1e30, so that f
+// is finite everywhere and such a hit is tested exactly against every candidate.
+// K slots: 0-7 -2ah.bh, 8-15 -2ah.bl, 16-23 -2al.bh, 24-26 |a|^2 parts x 1, 27-29 1 x |b|^2 parts.
 constexpr float kFrnnSlack = 1.0f / 16384.0f;
+constexpr float kFrnnWildNorm = 1e18f, kFrnnWild = -1e30f;
 
 __device__ __forceinline__ uint32_t frnn_hi(float x, float y) { return pack_bf16x2(x, y); }
 __device__ __forceinline__ uint32_t frnn_lo(float x, float y, uint32_t hi) {
@@ -130,12 +133,14 @@ __global__ void frnn_fragments_kernel(const float4* __restrict__ emb_s, int n, u
   }
   nb += __shfl_xor_sync(0xffffffffu, nb, 1);
   nb += __shfl_xor_sync(0xffffffffu, nb, 2);
-  nb = pos < n ? nb * (1.0f - kFrnnSlack) : 1e30f;
+  const bool wild = !(nb < kFrnnWildNorm);
+  nb = pos >= n ? -kFrnnWild : wild ? kFrnnWild : nb * (1.0f - kFrnnSlack);
   float q[3];
   frnn_parts(nb, q);
 #pragma unroll
   for (int s = 0; s < SETS; ++s) {
     uint4 w;
+    if (wild) v[s] = make_float2(0.f, 0.f);
     w.x = frnn_hi(v[s].x, v[s].y);
     w.y = frnn_lo(v[s].x, v[s].y, w.x);
     w.z = s > 0 ? 0u : t == 0 ? pack_bf16x2(1.f, 1.f) : t == 1 ? pack_bf16x2(1.f, q[0]) : t == 2 ? pack_bf16x2(q[1], q[2]) : 0u;
@@ -144,17 +149,12 @@ __global__ void frnn_fragments_kernel(const float4* __restrict__ emb_s, int n, u
   }
 }
 
+// D = A B + C, bf16 operands, fp32 accumulators.
 __device__ __forceinline__ void mma_m16n8k16(float* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                             uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ float min_nan(float a, float b) {       // NaN when either is
-  float m;
-  asm("min.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
-  return m;
+                                             uint32_t b1, const float* c) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 
 __device__ __forceinline__ float frnn_acc(float s, float a, float b) {
@@ -213,68 +213,121 @@ __global__ void __launch_bounds__(256) frnn_copy_kernel(const float* __restrict_
 // sorted positions from two cells below the first query's to two above the last one's.  (A run wider
 // than a query's own five cells holds no further partners of it, only pairs the exact test turns down.)
 // The filter takes the run eight candidates and sixteen queries at a time, 32 candidates between
-// votes; a vote that finds candidates tests them exactly and hands each query's partners, in ascending
-// position, to the lane that keeps its list.  One thread per hit with the exact test on every candidate
-// took 24 fp32 operations a pair (3.5e9 pairs on the full event, D = 8); the filter takes two MMAs and
-// about five other warp instructions for 128 pairs.  The build of the full event: 4.25 -> 1.07 ms, of which
-// this kernel takes 0.86.
+// votes.  The pairs it lets through wait in a queue, in ascending position for each query, until there
+// are 32 for the warp's lanes to test exactly and append to the queries' lists.
+//
+// The bound is the filter's instructions and the latency of its MMAs: on the full event (D = 8, 2.5e9 pairs
+// in the runs, 1.2e6 edges) 22 warp instructions for 128 pairs, two of them MMAs, with 28 warps per SM.  With
+// one thread per hit and the exact test on every candidate the search took 24 fp32 operations a pair, 3.2-4.2
+// ms; with each block's survivors tested on the spot by the lanes that held them 0.86 ms, queued 0.80, and with
+// 72 registers instead of 96 (seven blocks per SM) 0.74.  32 queries per warp test more pairs than they save
+// loads (0.77-0.85).
 constexpr int kFrnnPairsThreads = 128;
 constexpr int kFrnnQueries = 16;
 constexpr int kFrnnBlockQueries = kFrnnPairsThreads / 32 * kFrnnQueries;
+constexpr int kFrnnQueue = 32 + 8 * kFrnnQueries;                       // below 32 left over, and one block's
 
 template <int CH, int K>
-__global__ void __launch_bounds__(kFrnnPairsThreads) frnn_pairs_kernel(
+__global__ void __launch_bounds__(kFrnnPairsThreads, 7) frnn_pairs_kernel(
     const float4* __restrict__ emb_s, const uint4* __restrict__ frag, const float* __restrict__ r_s, int n, float r2,
     int grid, const int* __restrict__ cell_keys, const int* __restrict__ ids, const int* __restrict__ cell_start,
     int write, int* __restrict__ counts, const int* __restrict__ total, int capacity, int32_t* __restrict__ out,
     int* __restrict__ chunks, int* __restrict__ next_chunk, int max_extra, uint32_t* err) {
   constexpr int SETS = (CH + 1) / 2;
   constexpr int W = 2 * kFrnnReach + 1;
-  constexpr int ROWS = K == 4 ? (W * W * W + 1) / 2 : (W * W + 1) / 2;   // rows at or after the queries' own
   constexpr int UNROLL = 4;                                              // blocks of eight candidates per vote
   constexpr unsigned FULL = 0xffffffffu;
+  struct Warp {
+    int pos[kFrnnQueue];                           // queued pairs: the candidate's sorted position, and
+    unsigned char query[kFrnnQueue];               // the query
+    int found[kFrnnQueries];                       // per query: partners so far (writing pass: next output slot)
+    int cur[kFrnnQueries];                         // the chunk being filled
+    int lost[kFrnnQueries];
+  };
+  __shared__ Warp warps[kFrnnPairsThreads / 32];
+  Warp& w = warps[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31, g = lane >> 2, q = lane & 3;
+  const unsigned below = (1u << lane) - 1u;
   const int t0 = (blockIdx.x * (kFrnnPairsThreads / 32) + (threadIdx.x >> 5)) * kFrnnQueries;
   if (t0 >= n) return;
-  // lanes 4g and 4g + 1 keep the lists of queries g and g + 8
-  const int mine = t0 + g + 8 * (q & 1);
-  bool want = q < 2 && mine < n;
-  int pos = 0, n_total = 0, i = 0;
-  float ri = 0.f;
+  bool want = lane < kFrnnQueries && t0 + lane < n;                     // lane < 16: query t0 + lane is searched for
+  int n_total = 0;
   if (write) {
     n_total = *total;
     if (n_total > capacity) {
       if (t0 == 0 && lane == 0) atomicOr(err, DEV_ERR_CAPACITY);
       return;
     }
-    want = want && chunks[(size_t)mine * kFrnnChunk + kFrnnChunk - 1] == kFrnnLost;   // the others: frnn_copy_kernel's
+    want = want && chunks[(size_t)(t0 + lane) * kFrnnChunk + kFrnnChunk - 1] == kFrnnLost;   // the others: frnn_copy_kernel's
     if (__ballot_sync(FULL, want) == 0u) return;
-    if (want) { pos = counts[mine]; i = ids[mine]; ri = r_s[mine]; }
   } else if (want) {
-    chunks[(size_t)mine * kFrnnChunk + kFrnnChunk - 1] = -1;         // link of the first chunk: none yet
+    chunks[(size_t)(t0 + lane) * kFrnnChunk + kFrnnChunk - 1] = -1;   // link of the first chunk: none yet
   }
-  int cur = mine, fill = 0, found = 0;             // counting pass: the chain being filled
-  bool lost = false;
-  auto take = [&](int p) {                         // a partner of this lane's query
+  if (lane < kFrnnQueries) {
+    w.found[lane] = write && want ? counts[t0 + lane] : 0;
+    w.cur[lane] = t0 + lane;
+    w.lost[lane] = 0;
+  }
+  __syncwarp();
+
+  // The exact test of the first m <= 32 queued pairs, and the partners to their queries' lists.
+  auto drain = [&](int m) {
+    int pf = 0, qi = kFrnnQueries;
+    bool hit = false;
+    if (lane < m) {
+      pf = w.pos[lane];
+      qi = w.query[lane];
+      float s = 0.f;
+#pragma unroll
+      for (int k = 0; k < CH; ++k) {
+        const float4 x = emb_s[(size_t)(t0 + qi) * CH + k], y = emb_s[(size_t)pf * CH + k];
+        s = frnn_acc(s, x.x, y.x);
+        s = frnn_acc(s, x.y, y.y);
+        s = frnn_acc(s, x.z, y.z);
+        s = frnn_acc(s, x.w, y.w);
+      }
+      hit = s < r2;
+    }
+    const unsigned peers = __match_any_sync(FULL, hit ? qi : kFrnnQueries);       // this query's partners
+    const int rank = __popc(peers & below), cnt = __popc(peers), leader = __ffs(peers) - 1;
+    const int had = hit ? w.found[qi] : 0, at = had + rank;
     if (write) {
-      const int jj = ids[p];
-      const float rj = r_s[p];
-      const bool i_first = ri < rj || (ri == rj && i < jj);
-      out[pos] = i_first ? i : jj;
-      out[(size_t)n_total + pos] = i_first ? jj : i;
-      ++pos;
-      return;
+      if (hit) {
+        const int i = ids[t0 + qi], jj = ids[pf];
+        const float ri = r_s[t0 + qi], rj = r_s[pf];
+        const bool i_first = ri < rj || (ri == rj && i < jj);
+        out[at] = i_first ? i : jj;
+        out[(size_t)n_total + at] = i_first ? jj : i;
+      }
+    } else {
+      constexpr int C = kFrnnChunk - 1;            // entries per chunk
+      const int have = had > 0 ? (had - 1) / C : 0;                               // chunks filled or begun, less one
+      const int more = hit ? (had + cnt - 1) / C - have : 0;                      // chunks this batch begins
+      const int cur = hit ? w.cur[qi] : 0;
+      const bool gone = hit && w.lost[qi];
+      int base = 0;
+      if (hit && rank == 0 && more > 0 && !gone) {
+        base = atomicAdd(next_chunk, more);
+        if (base >= 0 && base <= max_extra - more) {
+          for (int k = 0, c = cur; k < more; c = n + base + k, ++k) chunks[(size_t)c * kFrnnChunk + C] = n + base + k;
+        } else {
+          base = -1;
+        }
+      }
+      base = __shfl_sync(FULL, base, leader);
+      const bool keep = hit && !gone && base >= 0;
+      if (keep) {
+        const int k = at / C - have;               // 0: the chunk being filled
+        chunks[(size_t)(k == 0 ? cur : n + base + k - 1) * kFrnnChunk + at % C] = pf;
+      }
+      if (hit && rank == 0) {
+        if (keep && more > 0) w.cur[qi] = n + base + more - 1;
+        if (base < 0) w.lost[qi] = 1;
+      }
     }
-    ++found;
-    if (lost) return;
-    if (fill == kFrnnChunk - 1) {
-      const int nc = atomicAdd(next_chunk, 1);
-      if (nc >= max_extra) { lost = true; return; }
-      chunks[(size_t)cur * kFrnnChunk + kFrnnChunk - 1] = n + nc;
-      cur = n + nc;
-      fill = 0;
-    }
-    chunks[(size_t)cur * kFrnnChunk + fill++] = p;
+    __syncwarp();                                  // every lane has read found and cur
+    if (hit && rank == 0) w.found[qi] = had + cnt;
+    __syncwarp();
   };
 
   // A fragments of queries g and g + 8: rows r = 0, 1
@@ -282,127 +335,170 @@ __global__ void __launch_bounds__(kFrnnPairsThreads) frnn_pairs_kernel(
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int t = t0 + g + 8 * r < n ? t0 + g + 8 * r : n - 1;
+    float2 v[SETS];
     float na = 0.f;
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
-      float2 v = make_float2(0.f, 0.f);
-      if (8 * s + 2 * q < 4 * CH) v = reinterpret_cast<const float2*>(emb_s)[(size_t)t * (2 * CH) + 4 * s + q];
-      na = fmaf(v.x, v.x, fmaf(v.y, v.y, na));
-      ah[s][r] = frnn_hi(-2.f * v.x, -2.f * v.y);
-      al[s][r] = frnn_lo(-2.f * v.x, -2.f * v.y, ah[s][r]);
+      v[s] = make_float2(0.f, 0.f);
+      if (8 * s + 2 * q < 4 * CH) v[s] = reinterpret_cast<const float2*>(emb_s)[(size_t)t * (2 * CH) + 4 * s + q];
+      na = fmaf(v[s].x, v[s].x, fmaf(v[s].y, v[s].y, na));
     }
     na += __shfl_xor_sync(FULL, na, 1);
     na += __shfl_xor_sync(FULL, na, 2);
-    float w[3];
-    frnn_parts(na * (1.0f - kFrnnSlack) - (r2 * (1.0f + 1.0f / 4096.0f) + 1e-35f), w);
-    an[r] = q == 0 ? pack_bf16x2(w[0], w[1]) : q == 1 ? pack_bf16x2(w[2], 1.f) : q == 2 ? pack_bf16x2(1.f, 1.f) : 0u;
+    const bool wild = !(na < kFrnnWildNorm);
+#pragma unroll
+    for (int s = 0; s < SETS; ++s) {
+      if (wild) v[s] = make_float2(0.f, 0.f);
+      ah[s][r] = frnn_hi(-2.f * v[s].x, -2.f * v[s].y);
+      al[s][r] = frnn_lo(-2.f * v[s].x, -2.f * v[s].y, ah[s][r]);
+    }
+    const float reach = fminf(r2 * (1.0f + 1.0f / 4096.0f) + 1e-35f, 1e29f);
+    float u[3];
+    frnn_parts(wild ? kFrnnWild : na * (1.0f - kFrnnSlack) - reach, u);
+    an[r] = q == 0 ? pack_bf16x2(u[0], u[1]) : q == 1 ? pack_bf16x2(u[2], 1.f) : q == 2 ? pack_bf16x2(1.f, 1.f) : 0u;
   }
-  const float4* ea[2] = {emb_s + (size_t)(t0 + g) * CH, emb_s + (size_t)(t0 + g + 8) * CH};
 
-  // the candidates of one block whose filter value c is not clearly beyond the radius
-  auto test_block = [&](const float* c, int blk, int p, int p1, const bool* member) {
-    uint32_t hits[2] = {0u, 0u};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int r = e >> 1, pf = 8 * blk + 2 * q + (e & 1);
-      if (!(c[e] >= 0.f) && member[r] && pf >= p && pf < p1 && pf > t0 + g + 8 * r) {
-        float s = 0.f;
-#pragma unroll
-        for (int k = 0; k < CH; ++k) {
-          const float4 x = ea[r][k], y = emb_s[(size_t)pf * CH + k];
-          s = frnn_acc(s, x.x, y.x);
-          s = frnn_acc(s, x.y, y.y);
-          s = frnn_acc(s, x.z, y.z);
-          s = frnn_acc(s, x.w, y.w);
-        }
-        hits[r] |= (s < r2 ? 1u : 0u) << (2 * q + (e & 1));
+  // Queries by row of cells (their keys ascend, so a row's queries are consecutive).  A row at level v is
+  // the cells that agree in all but the last v + 1 gridded coordinates; its runs reach two cells beyond the
+  // queries' first of those coordinates and over all of the others.  Level 0 tests the fewest pairs.  Where
+  // hits are sparse a warp's queries lie in many rows, each with a search of its own for a handful of
+  // candidates; a coarser level then puts them into fewer rows with longer runs.
+  const int slot = lane & (kFrnnQueries - 1);
+  const int key = cell_keys[t0 + slot < n ? t0 + slot : n - 1];
+  const unsigned wanted = __ballot_sync(FULL, want);
+  auto groups_at = [&](int d1) {                   // rows among the wanted queries, d1 = cells per row
+    const int gid = key / d1, prev = __shfl_up_sync(FULL, gid, 1);
+    return __popc(__ballot_sync(FULL, lane == 0 || gid != prev) & wanted) + ((wanted & 1u) ? 0 : 1);
+  };
+  // the run of this lane's row of cells (o-th at or after the queries' own), for queries first..last
+  auto row_run = [&](int level, int d0, int d1, int first, int last, int o, int& p, int& p1) {
+    const int gid = __shfl_sync(FULL, key / d1, first);
+    const int c_lo = __shfl_sync(FULL, (key / d0) % grid, first) - kFrnnReach;
+    const int c_hi = __shfl_sync(FULL, (key / d0) % grid, last) + kFrnnReach;
+    p = p1 = 0;
+    int rows = 1;
+    for (int k = level + 1; k < K; ++k) rows *= W;
+    if (o >= (rows + 1) / 2) return;
+    int l = rows / 2 + o, rest = gid, row = 0, scale = 1;
+    bool in = true;
+    for (int k = level + 1; k < K; ++k) {
+      const int c = rest % grid + l % W - kFrnnReach;
+      in = in && c >= 0 && c < grid;
+      row += c * scale;
+      rest /= grid; l /= W; scale *= grid;
+    }
+    if (!in) return;
+    const int lo = (c_lo < 0 ? 0 : c_lo) * d0, hi = (c_hi >= grid ? grid : c_hi + 1) * d0;
+    p = o == 0 ? t0 + first + 1 : cell_start[row * d1 + lo];
+    p1 = cell_start[row * d1 + hi];
+  };
+  int level = 0, d0 = 1;
+  const int fine = groups_at(grid);
+  if (fine > 2) {
+    // A coarser level costs its MMAs, found from its first row's runs; level 0 about 120 MMAs' time per
+    // row of cells (63 rows looked up, a few runs of four MMAs and their set-up).  Taken when it is cheaper,
+    // the finest first.  With level 0 throughout, 2,000 hits took 187 us and 30,000 took 234.
+    for (int v = 1, e0 = grid; v < K; ++v, e0 *= grid) {
+      const int e1 = e0 * grid, gs = groups_at(e1);
+      const int first = __ffs(wanted) - 1;
+      const unsigned same = __ballot_sync(FULL, key / e1 == __shfl_sync(FULL, key / e1, first)) & wanted;
+      int p, p1;
+      row_run(v, e0, e1, first, 31 - __clz(same), lane, p, p1);
+      const int blocks = p < p1 ? (p1 - p) / 8 + 6 : 0;
+      if ((long long)gs * (__reduce_add_sync(FULL, blocks) + 40) < 120LL * fine) {
+        level = v;
+        d0 = e0;
+        break;
       }
     }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {                  // the quad's eight candidates of each query
-      hits[r] |= __shfl_xor_sync(FULL, hits[r], 1);
-      hits[r] |= __shfl_xor_sync(FULL, hits[r], 2);
-    }
-    if (q < 2)
-      for (uint32_t m = hits[q]; m; m &= m - 1) take(8 * blk + __ffs(m) - 1);
-  };
-
-  // queries by row of cells (their keys ascend, so a row's queries are consecutive)
-  const int key = cell_keys[t0 + (lane & 15) < n ? t0 + (lane & 15) : n - 1];
-  const int row = key / grid, cl = key - row * grid;
-  const bool wa = __shfl_sync(FULL, want, (lane & 7) * 4 + ((lane >> 3) & 1));      // query lane & 15 is wanted
-  unsigned todo = __ballot_sync(FULL, wa && lane < 16);
+  }
+  const int d1 = d0 * grid;
+  int rows = 1;
+  for (int k = level + 1; k < K; ++k) rows *= W;
+  rows = (rows + 1) / 2;
+  unsigned todo = wanted;
+  int queued = 0;
   while (todo) {
     const int first = __ffs(todo) - 1;
-    const int rid = __shfl_sync(FULL, row, first);
-    const unsigned same = __ballot_sync(FULL, row == rid) & todo;
+    const unsigned same = __ballot_sync(FULL, key / d1 == __shfl_sync(FULL, key / d1, first)) & todo;
     todo &= ~same;
     const int last = 31 - __clz(same);
-    const int c_lo = __shfl_sync(FULL, cl, first) - kFrnnReach, c_hi = __shfl_sync(FULL, cl, last) + kFrnnReach;
-    const int lo = c_lo < 0 ? 0 : c_lo, hi = c_hi >= grid ? grid - 1 : c_hi;
-    const bool member[2] = {((same >> g) & 1u) != 0u, ((same >> (g + 8)) & 1u) != 0u};
-    for (int base = 0; base < ROWS; base += 32) {
-      // one row of cells per lane: its run of sorted positions
-      int p = 0, p1 = 0;
-      const int o = base + lane;
-      if (o < ROWS) {
-        const int l = (K == 4 ? (W * W * W) / 2 : (W * W) / 2) + o;
-        int ra, rb, rc = 0, rr;
-        bool in;
-        if constexpr (K == 4) {
-          ra = rid / (grid * grid) + l / (W * W) - kFrnnReach;
-          rb = (rid / grid) % grid + (l / W) % W - kFrnnReach;
-          rc = rid % grid + l % W - kFrnnReach;
-          in = ra < grid && rb >= 0 && rb < grid && rc >= 0 && rc < grid;
-          rr = (ra * grid + rb) * grid + rc;
-        } else {
-          ra = rid / grid + l / W - kFrnnReach;
-          rb = rid % grid + l % W - kFrnnReach;
-          in = ra < grid && rb >= 0 && rb < grid;
-          rr = ra * grid + rb;
-        }
-        if (in) {
-          p = o == 0 ? t0 + first + 1 : cell_start[rr * grid + lo];
-          p1 = cell_start[rr * grid + hi + 1];
-        }
-      }
+    bool member[2];
+    uint32_t norm[2];                              // a query of another row: a norm that no radius reaches
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      member[r] = ((same >> (g + 8 * r)) & 1u) != 0u;
+      norm[r] = member[r] ? an[r] : q == 0 ? pack_bf16x2(-kFrnnWild, 0.f) : q == 1 ? pack_bf16x2(0.f, 1.f) : an[r];
+    }
+    for (int base = 0; base < rows; base += 32) {
+      int p, p1;                                   // one row of cells per lane: its run of sorted positions
+      row_run(level, d0, d1, first, last, base + lane, p, p1);
       for (unsigned runs = __ballot_sync(FULL, p < p1); runs; runs &= runs - 1) {
         const int from = __ffs(runs) - 1;
         const int rp = __shfl_sync(FULL, p, from), rp1 = __shfl_sync(FULL, p1, from);
         const int b1 = (rp1 + 7) >> 3;
         for (int b = rp >> 3; b < b1; b += UNROLL) {
           float c[UNROLL][4];
-          float m = 0.f;
+          uint32_t neg = 0u;                       // sign bits
 #pragma unroll
           for (int u = 0; u < UNROLL; ++u) {
             const int blk = b + u < b1 ? b + u : b1 - 1;             // past the run's end: its last block again
             const uint4* f = frag + (size_t)blk * (32 * SETS) + lane;
-            const uint4 w = f[0];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) c[u][e] = 0.f;
-            mma_m16n8k16(c[u], ah[0][0], ah[0][1], ah[0][0], ah[0][1], w.x, w.y);
-            mma_m16n8k16(c[u], al[0][0], al[0][1], an[0], an[1], w.x, w.z);
+            const uint4 x = f[0];
+            const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_m16n8k16(c[u], ah[0][0], ah[0][1], ah[0][0], ah[0][1], x.x, x.y, zero);
+            mma_m16n8k16(c[u], al[0][0], al[0][1], norm[0], norm[1], x.x, x.z, c[u]);
             if constexpr (SETS == 2) {
-              const uint4 w2 = f[32];
-              mma_m16n8k16(c[u], ah[1][0], ah[1][1], ah[1][0], ah[1][1], w2.x, w2.y);
-              mma_m16n8k16(c[u], al[1][0], al[1][1], 0u, 0u, w2.x, 0u);
+              const uint4 y = f[32];
+              mma_m16n8k16(c[u], ah[1][0], ah[1][1], ah[1][0], ah[1][1], y.x, y.y, c[u]);
+              mma_m16n8k16(c[u], al[1][0], al[1][1], 0u, 0u, y.x, 0u, c[u]);
             }
-            m = min_nan(m, min_nan(min_nan(c[u][0], c[u][1]), min_nan(c[u][2], c[u][3])));
+            neg |= __float_as_uint(c[u][0]) | __float_as_uint(c[u][1]);
+            neg |= __float_as_uint(c[u][2]) | __float_as_uint(c[u][3]);
           }
-          if (__any_sync(FULL, !(m >= 0.f))) {
+          if (!__any_sync(FULL, (int)neg < 0)) continue;
 #pragma unroll
-            for (int u = 0; u < UNROLL; ++u) {
-              const float mu = min_nan(min_nan(c[u][0], c[u][1]), min_nan(c[u][2], c[u][3]));
-              if (b + u < b1 && __any_sync(FULL, !(mu >= 0.f))) test_block(c[u], b + u, rp, rp1, member);
+          for (int u = 0; u < UNROLL; ++u) {
+            const uint32_t any = __float_as_uint(c[u][0]) | __float_as_uint(c[u][1]) | __float_as_uint(c[u][2]) |
+                                 __float_as_uint(c[u][3]);
+            if (b + u >= b1 || !__any_sync(FULL, (int)any < 0)) continue;
+            // this block's pairs into the queue, by lane and then by column: ascending for each query
+            unsigned ball[4];
+            int before = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int r = e >> 1, pf = 8 * (b + u) + 2 * q + (e & 1);
+              ball[e] = __ballot_sync(FULL, c[u][e] < 0.f && member[r] && pf >= rp && pf < rp1 && pf > t0 + g + 8 * r);
+              before += __popc(ball[e] & below);
+            }
+            int at = queued + before;
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if ((ball[e] >> lane) & 1u) {
+                w.pos[at] = 8 * (b + u) + 2 * q + (e & 1);
+                w.query[at] = (unsigned char)(g + 8 * (e >> 1));
+                ++at;
+              }
+            queued += __popc(ball[0]) + __popc(ball[1]) + __popc(ball[2]) + __popc(ball[3]);
+            __syncwarp();
+            while (queued >= 32) {
+              drain(32);
+              queued -= 32;
+              for (int k = lane; k < queued; k += 32) {              // the rest to the front (a lane only
+                w.pos[k] = w.pos[32 + k];                            // writes where it alone has read)
+                w.query[k] = w.query[32 + k];
+              }
+              __syncwarp();
             }
           }
         }
       }
     }
   }
+  if (queued > 0) drain(queued);
   if (!write && want) {
-    counts[mine] = found;
-    if (lost) chunks[(size_t)mine * kFrnnChunk + kFrnnChunk - 1] = kFrnnLost;
+    counts[t0 + lane] = w.found[lane];
+    if (w.lost[lane]) chunks[(size_t)(t0 + lane) * kFrnnChunk + kFrnnChunk - 1] = kFrnnLost;
   }
 }
 
