@@ -83,6 +83,7 @@ template <typename Src>
 __global__ void __launch_bounds__(kRadixThreads) radix_count_kernel(const Src src, int n, int shift, int bins, int n_tiles,
                                                                     int* __restrict__ hist) {
   pdl_wait();
+  pdl_trigger_small();
   __shared__ int cnt[kRadixMaxBins];
   for (int d = threadIdx.x; d < bins; d += kRadixThreads) cnt[d] = 0;
   __syncthreads();
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(kRadixThreads) radix_count_kernel(const Src sr
 __global__ void __launch_bounds__(kRadixThreads) radix_scan_kernel(int* __restrict__ hist, int bins, int n_tiles,
                                                                    int* __restrict__ totals) {
   pdl_wait();
+  pdl_trigger_small();
   const int d = blockIdx.x * kRadixWarps + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (d >= bins) return;
   int* h = hist + (size_t)d * n_tiles;
@@ -138,6 +140,7 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src 
                                                                       const int* __restrict__ offs,
                                                                       const int* __restrict__ totals) {
   pdl_wait();
+  pdl_trigger_small();
   __shared__ int first[kRadixMaxBins];                     // global position of the tile's first element per digit
   __shared__ uint16_t wcnt[kRadixWarps][kRadixMaxBins];
   __shared__ int wsum[kRadixWarps];
@@ -218,6 +221,7 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src 
 __global__ void csr_rowptr_kernel(const int* __restrict__ keys_sorted, int n_edges, int n_nodes,
                                   int* __restrict__ rowptr) {
   pdl_wait();
+  pdl_trigger_small();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > n_nodes) return;
   int lo = 0, hi = n_edges;
@@ -234,6 +238,7 @@ __global__ void csr_finish_kernel(const int32_t* __restrict__ ei, const int* __r
                                   const int* __restrict__ vals_sorted, int n_edges, int n_nodes, int* __restrict__ perm,
                                   int* __restrict__ src_sorted, int* __restrict__ dst_sorted, int* __restrict__ rowptr) {
   pdl_wait();
+  pdl_trigger_small();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_edges) {
     const int id = vals_sorted[i], key = keys_sorted[i];

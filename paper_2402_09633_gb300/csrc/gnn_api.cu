@@ -416,6 +416,7 @@ cudaError_t launch_tile(gnn_ctx* c, const KernelPlan& pl, TileParams p, cudaStre
   if (p.n_tiles == 0) return cudaSuccess;
   const uint32_t smem = tile_launch_smem<H, BF>(p.n_vec_floats, p.const_bytes);
   const int grid = tile_grid(p.n_tiles, c->n_sm);
+  p.early = 2 * grid <= c->n_sm;
 #ifdef GNN_TRACE
   p.trace = ((int)K == c->trace_kind) ? c->trace : nullptr;
 #endif

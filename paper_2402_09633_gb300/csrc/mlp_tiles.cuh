@@ -95,6 +95,7 @@ struct TileParams {
   int job_acc[kMaxJobs];      // 1: accumulate into D (second half of a split layer 1)
   int job_areg[kMaxJobs];     // two groups: which of the group's two regions holds A (D is the other)
   int job_bias[kMaxJobs];     // bias tile (1-based, into consts) that the job's D starts from; 0: none
+  int early;                  // 1: a small grid, let the next kernel start on the idle SMs (see pdl_trigger)
   int folded;                 // 1: gamma of every layer but the MLP's last is folded into the weights around it
   const uint8_t* consts;      // the ones tile, then the bias tiles (128 and H rows x 16 bf16, see gnn_api.cu)
   uint32_t const_bytes;
@@ -252,6 +253,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
   // no earlier kernel, so under a programmatic dependent launch it overlaps the previous kernel's
   // exit; from here on every thread may read what that kernel wrote.
   pdl_wait();
+  if (p.early) pdl_trigger();
   GNN_TRACE_CTA(0);
 
   if (warp == 0) {
@@ -994,6 +996,7 @@ __global__ void __launch_bounds__(256) aggregate_kernel(const void* __restrict__
   const SE* e = static_cast<const SE*>(e_);
   SE* agg = static_cast<SE*>(agg_);
   pdl_wait();
+  pdl_trigger_small();
   const int li = threadIdx.x % LPN;
   const int bp = li >> 2, q = li & 3;
   const int j = n_nodes - 1 - (blockIdx.x * agg_nodes_per_block<H>() + (int)threadIdx.x / LPN);

@@ -207,11 +207,18 @@ __device__ __forceinline__ void tmem_st_wait() {
 // Programmatic dependent launch: the executing thread waits until every grid this one depends on has
 // completed and its memory writes are visible (it returns at once when the kernel was not launched
 // as a programmatic dependent).  Everything a kernel does before it may overlap the previous kernel,
-// so it must touch no data that kernel writes or reads.  The kernels here issue no early launch
-// trigger (griddepcontrol.launch_dependents): a dependent then launches as its predecessor's CTAs
-// exit, which hides the launch latency; measured on the full event, 6.59 -> 6.51 ms per step, while
-// triggering at the start or at the end of a tile kernel's work made it 6.83 ms.
+// so it must touch no data that kernel writes or reads.  Without a trigger a dependent launches as its
+// predecessor's CTAs exit, which hides the launch latency.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the next kernel's CTAs launch as soon as every CTA of this one has called it (after its own
+// pdl_wait), where SMs are free; they set up (weights, tensor memory, barriers) and wait.  Worth it only
+// when this grid leaves SMs idle: tiny event (57 CTAs) 120 -> 114 us, 3,000 hits / 9,000 edges 195 -> 188; with
+// tile kernels that fill every SM it made the full event's step slower (6.51 -> 6.83 ms, an earlier form of
+// the kernels) and the mid event's (716 -> 726 us).
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger_small() {
+  if (gridDim.x <= 64) pdl_trigger();
+}
 
 // ------------------------------------------------- 32-byte global accesses
 // One 32-byte sector per thread (256-bit accesses, sm_100 and later; the address is 32-byte aligned).
