@@ -414,7 +414,9 @@ cudaError_t launch_tile(gnn_ctx* c, const KernelPlan& pl, TileParams p, cudaStre
   p.mat_bytes = c->mat_bytes;
   p.n_tiles = (p.n_rows + kTileRows - 1) / kTileRows;
   if (p.n_tiles == 0) return cudaSuccess;
-  const uint32_t smem = tile_launch_smem<H, BF>(p.n_vec_floats, p.const_bytes);
+  const int stages = tile_stages<K, H, BF>(p.n_jobs);
+  p.ring_bytes = stages * TileGeom<H, BF>::MAT_BYTES;
+  const uint32_t smem = tile_launch_smem<H, BF>(stages, p.n_vec_floats, p.const_bytes);
   const int grid = tile_grid(p.n_tiles, c->n_sm);
   p.early = 2 * grid <= c->n_sm;
 #ifdef GNN_TRACE

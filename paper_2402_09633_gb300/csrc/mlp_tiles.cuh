@@ -99,6 +99,7 @@ struct TileParams {
   int folded;                 // 1: gamma of every layer but the MLP's last is folded into the weights around it
   const uint8_t* consts;      // the ones tile, then the bias tiles (128 and H rows x 16 bf16, see gnn_api.cu)
   uint32_t const_bytes;
+  uint32_t ring_bytes;        // weight ring (a stage per job where all jobs' weights fit)
   const uint8_t* wmats;       // packed matrices, mat_bytes apart (hi part then lo part)
   uint32_t mat_bytes;
   const float* vecs;          // per-kernel fp32 parameter vectors (layout per kind)
@@ -154,8 +155,7 @@ struct TileGeom {
   static constexpr int NREG = TMEM_COLS / H;        // regions: 4 (H = 128) or 8 (H = 64)
   static constexpr uint32_t PART_BYTES = H * H * 2; // one bf16 H x H matrix part
   static constexpr uint32_t MAT_BYTES = BF ? PART_BYTES : 2 * PART_BYTES;  // hi [+ lo]
-  static constexpr int STAGES = (192u * 1024u / MAT_BYTES) < 8 ? (192u * 1024u / MAT_BYTES) : 8;  // weight ring depth
-  static constexpr uint32_t RING_BYTES = STAGES * MAT_BYTES;
+  static constexpr int STAGES = (192u * 1024u / MAT_BYTES) < 8 ? (192u * 1024u / MAT_BYTES) : 8;  // weight ring, at most
   static constexpr uint32_t IDESC = idesc_bf16_f32(128, H);
   static constexpr uint32_t ONES_BYTES = 128 * 32;  // 128 rows x 16 bf16
   static constexpr uint32_t BIAS_BYTES = H * 32;    // H rows x 16 bf16
@@ -171,18 +171,39 @@ __host__ __device__ constexpr uint32_t input_part_offset(int w) {
 // Parameter vectors are padded to 16 bytes so the mbarriers after them stay 8-byte aligned.
 __host__ __device__ constexpr int padded_vec_floats(int n) { return (n + 3) & ~3; }
 
+// Stages of a kernel's weight ring, at most; weights that need no more stay resident.  The node kernels of
+// H = 128 stream their five to seven blocks through a shorter ring than would fit (two blocks in fp32, four in
+// bf16): the L1 that it leaves is worth more (node update 0.179 -> 0.170 ms and 0.127 -> 0.118; a bf16 ring of
+// five or three 0.127).
+template <TileKind KIND, int H, bool BF>
+constexpr int tile_max_stages() {
+  constexpr int most = TileGeom<H, BF>::STAGES;
+  if (H == 128 && (KIND == TileKind::NodeUpdate || KIND == TileKind::NodeEncoder)) return BF ? 4 : 2;
+  return most;
+}
+// Stages taken: one per job where they all fit, no more.  Shared memory that is not taken is L1: next to the
+// full 192 KB it has about 230 lines left, too few for the loads that the worker warps have in flight (bf16
+// edge update 0.240 -> 0.210 ms with 96 KB of weights instead of a 192 KB ring).  The fp32 kernels of H = 128
+// need the full ring for three layers; they keep it, at a fixed offset, for two (a computed offset costs the
+// edge update spills: 0.318 -> 0.338).
+template <TileKind KIND, int H, bool BF>
+constexpr int tile_stages(int n_jobs) {
+  constexpr int most = tile_max_stages<KIND, H, BF>();
+  return n_jobs < most && !(H == 128 && !BF) ? n_jobs : most;
+}
+
 template <int H, bool BF>
-constexpr uint32_t tile_smem_bytes(int n_vec_floats, uint32_t const_bytes) {
+constexpr uint32_t tile_smem_bytes(int stages, int n_vec_floats, uint32_t const_bytes) {
   // ring (1024-aligned) + ones and bias tiles + vectors + barriers + alignment slack
-  return TileGeom<H, BF>::RING_BYTES + const_bytes + (uint32_t)padded_vec_floats(n_vec_floats) * 4u + 320 + 1024;
+  return stages * TileGeom<H, BF>::MAT_BYTES + const_bytes + (uint32_t)padded_vec_floats(n_vec_floats) * 4u + 320 + 1024;
 }
 
 // Launch geometry: dynamic shared memory of at least 120 KB, so that one CTA per SM runs (it owns
 // the TMEM), and one persistent CTA per SM or per tile, whichever is fewer.  CTA b takes tiles b,
 // b + grid, b + 2 grid, ...; its groups take them in turn.
 template <int H, bool BF>
-constexpr uint32_t tile_launch_smem(int n_vec_floats, uint32_t const_bytes) {
-  const uint32_t b = tile_smem_bytes<H, BF>(n_vec_floats, const_bytes);
+constexpr uint32_t tile_launch_smem(int stages, int n_vec_floats, uint32_t const_bytes) {
+  const uint32_t b = tile_smem_bytes<H, BF>(stages, n_vec_floats, const_bytes);
   return b < 120u * 1024u ? 120u * 1024u : b;
 }
 inline int tile_grid(int n_tiles, int n_sm) { return n_tiles < n_sm ? n_tiles : n_sm; }
@@ -202,11 +223,12 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
   using R = TileRoles<KIND>;
   constexpr int NG = R::NG;
   constexpr int NCH = G::NCH;
+  constexpr int STAGES = tile_max_stages<KIND, H, BF>();
   constexpr int NSPARE = G::NREG - NG;               // regions no group owns (three groups)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* ring = smem;
-  uint8_t* consts = smem + G::RING_BYTES;
+  uint8_t* consts = smem + (H == 128 && !BF ? STAGES * G::MAT_BYTES : p.ring_bytes);
   float* vecs = reinterpret_cast<float*>(consts + p.const_bytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(vecs + padded_vec_floats(p.n_vec_floats));
   uint64_t* a_full = bars;                           // [3]  a group's eight warps published A
@@ -214,14 +236,14 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
   uint64_t* spare_free = bars + 6;                   // [8]  the job that gave a spare region back completed
   uint64_t* c_full = bars + 14;                      // the constant tiles are loaded
   uint64_t* w_full = bars + 15;                      // [STAGES]  weight stage loaded
-  uint64_t* w_empty = bars + 15 + G::STAGES;         // [STAGES]  all groups' MMAs on a stage completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 15 + 2 * G::STAGES);
+  uint64_t* w_empty = bars + 15 + STAGES;         // [STAGES]  all groups' MMAs on a stage completed
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 15 + 2 * STAGES);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   volatile int* d_region = abort_flag + 1;           // [3]  three groups: the region of a group's current D
 
   const int warp = uniform((int)threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
-  const bool resident = p.n_jobs <= G::STAGES;
+  const bool resident = p.n_jobs <= STAGES;
   const int n_my = (p.n_tiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // this CTA's tiles
   const int n_rounds = (n_my + NG - 1) / NG;
 
@@ -232,7 +254,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
       mbar_init(&d_full[g], NG == 3 ? 2 : 1);        // three groups: the commit, and the issuer's region word
     }
     for (int s = 0; s < 8; ++s) mbar_init(&spare_free[s], 1);
-    for (int s = 0; s < G::STAGES; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], NG); }
+    for (int s = 0; s < STAGES; ++s) { mbar_init(&w_full[s], 1); mbar_init(&w_empty[s], NG); }
     mbar_init(c_full, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -288,8 +310,8 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
     while (ok && live > 0) {
       bool progressed = false;
       if (loaded < to_load) {
-        const int st = loaded % G::STAGES;
-        if (loaded < (uint32_t)G::STAGES || warp_all(mbar_test_wait(&w_empty[st], ((loaded / G::STAGES) - 1) & 1))) {
+        const int st = loaded % STAGES;
+        if (loaded < (uint32_t)STAGES || warp_all(mbar_test_wait(&w_empty[st], ((loaded / STAGES) - 1) & 1))) {
           const uint8_t* src = p.wmats + (size_t)p.job_mat[loaded % p.n_jobs] * p.mat_bytes;
           if (elect_one()) {
             mbar_arrive_expect_tx(&w_full[st], G::MAT_BYTES);
@@ -304,8 +326,8 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
       for (int g = 0; g < NG; ++g) {
         if (i_g[g] >= n_my) continue;
         const int j = job_g[g];
-        const int st = resident ? j : (int)(seq_g[g] % G::STAGES);
-        if (!resident && !warp_all(mbar_test_wait(&w_full[st], (seq_g[g] / G::STAGES) & 1))) continue;
+        const int st = resident ? j : (int)(seq_g[g] % STAGES);
+        if (!resident && !warp_all(mbar_test_wait(&w_full[st], (seq_g[g] / STAGES) & 1))) continue;
         if (!warp_all(mbar_test_wait(&a_full[g], a_par[g]))) continue;
         a_par[g] ^= 1;
         uint32_t ra, rd;
@@ -396,8 +418,8 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
     // ... and every weight copy has landed (the last one per stage)
     drain_wait(c_full, 0);
     if (resident) drain_wait(&w_full[0], 0);
-    for (uint32_t k = loaded > (uint32_t)G::STAGES ? loaded - G::STAGES : 0u; k < loaded; ++k)
-      drain_wait(&w_full[k % G::STAGES], (k / G::STAGES) & 1);
+    for (uint32_t k = loaded > (uint32_t)STAGES ? loaded - STAGES : 0u; k < loaded; ++k)
+      drain_wait(&w_full[k % STAGES], (k / STAGES) & 1);
     __syncwarp();
   } else {
     // Worker groups: eight warps to a group, sixteen rows of its tile to a warp (half of a tensor-memory
