@@ -79,7 +79,7 @@ __host__ __device__ constexpr bool has_input_job(TileKind k) {
 // Worker groups and threads of a kernel: one warp that issues, and eight per group.
 template <TileKind KIND>
 struct TileRoles {
-  static constexpr int NG = (KIND == TileKind::NodeEncoder || KIND == TileKind::NodeUpdate) ? 2 : 3;
+    static constexpr int NG = (KIND == TileKind::NodeEncoder || KIND == TileKind::NodeUpdate) ? 2 : 3;
   static constexpr int THREADS = 32 + 256 * NG;      // 800 (80 registers each) or 544 (120)
 };
 
@@ -174,11 +174,15 @@ __host__ __device__ constexpr int padded_vec_floats(int n) { return (n + 3) & ~3
 // Stages of a kernel's weight ring, at most; weights that need no more stay resident.  The node kernels of
 // H = 128 stream their five to seven blocks through a shorter ring than would fit (two blocks in fp32, four in
 // bf16): the L1 that it leaves is worth more (node update 0.179 -> 0.170 ms and 0.127 -> 0.118; a bf16 ring of
-// five or three 0.127).
+// five or three 0.127).  So is the fp32 edge update's and classifier's, whose gathers need it (three resident
+// blocks 0.319 and 0.291 ms, two streamed 0.298 and 0.265; mid event 704 -> 670 us); the kernels without
+// gathers keep three resident (filter 0.344, two streamed 0.366).  Stages of half a block (hi and lo parts
+// apart) were slower at every depth (0.303-0.331).
 template <TileKind KIND, int H, bool BF>
 constexpr int tile_max_stages() {
   constexpr int most = TileGeom<H, BF>::STAGES;
   if (H == 128 && (KIND == TileKind::NodeUpdate || KIND == TileKind::NodeEncoder)) return BF ? 4 : 2;
+  if (H == 128 && !BF && (KIND == TileKind::EdgeUpdate || KIND == TileKind::Classifier)) return 2;
   return most;
 }
 // Stages taken: one per job where they all fit, no more.  Shared memory that is not taken is L1: next to the
@@ -523,10 +527,11 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
         tmem_st_16x16(reg + 32 * c + 16, lo);
       }
     };
-    // Two T16 state rows -> A operand, AHEAD chunks of loads in flight (rows past the end lie in the
-    // buffers' padding to whole tiles).
+    // Two T16 state rows -> A operand, AHEAD chunks of loads in flight: whole rows in the two-group kernels
+    // (node update 0.170 -> 0.163 ms against three chunks), two chunks where registers are scarcer (edge update
+    // 0.295 -> 0.291).  Rows past the end lie in the buffers' padding to whole tiles.
     auto state_to_a = [&](uint32_t reg, const void* base, int row) {
-      constexpr int AHEAD = NCH < 3 ? NCH : 3;
+      constexpr int AHEAD = NCH < 2 * (4 - NG) ? NCH : 2 * (4 - NG);
       using V = typename std::conditional<BF, uint2, float4>::type;
       V m[NCH][4];
 #pragma unroll
@@ -790,7 +795,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
         GNN_TRACE_W(1);
         // layer-1 terms of the endpoints, loaded while the MMA runs: S = P_s[src] + P_d[dst] (P_d
         // carries b1), the first chunks before D is waited for, the others while those are added
-        constexpr int EARLY = NCH < 2 ? NCH : 2;
+                constexpr int EARLY = NCH < 2 ? NCH : 2;
         float2 S[NCH][8];
         auto gather = [&](int c) {
 #pragma unroll
