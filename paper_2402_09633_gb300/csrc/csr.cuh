@@ -19,7 +19,7 @@
 // and a dependent load each, one block walking every tile's counts.  Here a
 // thread's sixteen elements are loaded at once, a warp ranks its own 512 elements
 // against its own counters without a block barrier, and a warp per digit scans
-// the counts, in seven launches.  1M edges, 300k nodes: 131 -> 66 us; 7,200 edges, 2,000 nodes (one pass):
+// the counts, in seven launches.  1M edges, 300k nodes: 131 -> 66 us, 58 with tiles sorted before they are written; 7,200 edges, 2,000 nodes (one pass):
 // nine launches -> four, 45 us of the tiny event's 164 less.
 #pragma once
 #include <cstdint>
@@ -132,7 +132,8 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scan_kernel(int* __restri
 // Stable scatter of one pass.  Warp w of a tile's block owns the tile's elements [512 w, 512 w + 512) and
 // takes them 32 at a time in input order: an element's rank among its warp's equal digits is the warp's
 // count so far plus __match_any_sync.  Then the warps' counts are scanned per digit, on top of the digit's
-// offset: keys with a smaller digit, plus those with this digit in earlier tiles.
+// offset: keys with a smaller digit, plus those with this digit in earlier tiles.  The tile is put in digit
+// order in shared memory first, so that neighbouring threads write neighbouring places of a digit's run.
 template <typename Src>
 __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src src, int* __restrict__ keys_out,
                                                                       int* __restrict__ vals_out, int n, int shift,
@@ -142,8 +143,10 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src 
   pdl_wait();
   pdl_trigger_small();
   __shared__ int first[kRadixMaxBins];                     // global position of the tile's first element per digit
-  __shared__ uint16_t wcnt[kRadixWarps][kRadixMaxBins];
-  __shared__ int wsum[kRadixWarps];
+  __shared__ uint16_t start[kRadixMaxBins];                // place of it inside the sorted tile
+  __shared__ __align__(16) uint16_t wcnt[kRadixWarps][kRadixMaxBins];   // counts; later the sorted tile
+  __shared__ int wsum[2][kRadixWarps];
+  static_assert(sizeof(wcnt) == 2 * kRadixTile * sizeof(int), "the sorted tile takes the counts' place");
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int base = blockIdx.x * kRadixTile + warp * (32 * kRadixRounds) + lane;
   int key[kRadixRounds], val[kRadixRounds];
@@ -168,13 +171,13 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src 
     const int y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
-  if (lane == 31) wsum[warp] = x;
+  if (lane == 31) wsum[0][warp] = x;
   const int half = bins >> 1, half_bits = __ffs(half) - 1;      // two 16-bit counts per word
   for (int i = t; i < kRadixWarps * half; i += kRadixThreads)
     reinterpret_cast<uint32_t*>(wcnt[i >> half_bits])[i & (half - 1)] = 0u;
   __syncthreads();
   int run = x - sum;
-  for (int w = 0; w < warp; ++w) run += wsum[w];
+  for (int w = 0; w < warp; ++w) run += wsum[0][w];
 #pragma unroll
   for (int k = 0; k < kRadixMaxBins / kRadixThreads; ++k) {
     const int d = t * per + k;
@@ -197,24 +200,63 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const Src 
     __syncwarp();
   }
   __syncthreads();
-  for (int d = t; d < bins; d += kRadixThreads) {          // counts of the warps before
-    int c = 0;
+  int cnt = 0;                                             // this thread's digits: counts of the warps before
+  int own[kRadixMaxBins / kRadixThreads];
 #pragma unroll
-    for (int w = 0; w < kRadixWarps; ++w) {
-      const int v = wcnt[w][d];
-      wcnt[w][d] = (uint16_t)c;
-      c += v;
+  for (int k = 0; k < kRadixMaxBins / kRadixThreads; ++k) {
+    const int d = t * per + k;
+    own[k] = cnt;
+    if (k < per && d < bins) {
+      int c = 0;
+#pragma unroll
+      for (int w = 0; w < kRadixWarps; ++w) {
+        const int v = wcnt[w][d];
+        wcnt[w][d] = (uint16_t)c;
+        c += v;
+      }
+      cnt += c;
     }
   }
+  int y = cnt;                                             // ... and of the smaller digits
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int z = __shfl_up_sync(0xffffffffu, y, o);
+    if (lane >= o) y += z;
+  }
+  if (lane == 31) wsum[1][warp] = y;
   __syncthreads();
+  int before = y - cnt;
+  for (int w = 0; w < warp; ++w) before += wsum[1][w];
+#pragma unroll
+  for (int k = 0; k < kRadixMaxBins / kRadixThreads; ++k) {
+    const int d = t * per + k;
+    if (k < per && d < bins) start[d] = (uint16_t)(before + own[k]);
+  }
+  __syncthreads();
+  int place[kRadixRounds];
+#pragma unroll
+  for (int r = 0; r < kRadixRounds; ++r) {
+    const int d = (key[r] >> shift) & (bins - 1);
+    place[r] = key[r] >= 0 ? start[d] + wcnt[warp][d] + rank[r] : 0;
+  }
+  __syncthreads();                                         // the counts are read: their place takes the tile
+  int* tile_key = reinterpret_cast<int*>(&wcnt[0][0]);
+  int* tile_val = tile_key + kRadixTile;
 #pragma unroll
   for (int r = 0; r < kRadixRounds; ++r)
     if (key[r] >= 0) {
-      const int d = (key[r] >> shift) & (bins - 1);
-      const int pos = first[d] + wcnt[warp][d] + rank[r];
-      keys_out[pos] = key[r];
-      vals_out[pos] = val[r];
+      tile_key[place[r]] = key[r];
+      tile_val[place[r]] = val[r];
     }
+  __syncthreads();
+  const int64_t left = (int64_t)n - (int64_t)blockIdx.x * kRadixTile;
+  const int m = left < kRadixTile ? (int)left : kRadixTile;
+  for (int i = t; i < m; i += kRadixThreads) {
+    const int k = tile_key[i], d = (k >> shift) & (bins - 1);
+    const int pos = first[d] + (i - start[d]);
+    keys_out[pos] = k;
+    vals_out[pos] = tile_val[i];
+  }
 }
 
 // rowptr[j] = first sorted slot whose key >= j (binary search), for j in [0, n_nodes].
