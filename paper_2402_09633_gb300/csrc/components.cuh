@@ -8,7 +8,7 @@
 // labels canonical: independent of thread order and of the order of the
 // edges.  During the unions, path halving writes are plain stores; they race
 // benignly because every value written is an ancestor of the node.  The final
-// pass only reads the forest (see cc_flatten_kernel).
+// pass never raises an entry (see cc_flatten_kernel).
 #pragma once
 #include <cstdint>
 #include "ptx.cuh"
@@ -20,6 +20,7 @@ namespace gnn {
 constexpr uint64_t kUnionLimitNs = 1000000000ull;   // 1 s
 
 __global__ void cc_init_kernel(int32_t* parent, int n) {
+  pdl_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v < n) parent[v] = v;
 }
@@ -42,11 +43,12 @@ __device__ __forceinline__ int cc_find(int32_t* parent, int x, uint64_t t0) {
 // endpoint outside [0, n) and edges whose score is NaN or <= threshold are skipped.
 __global__ void cc_union_kernel(const float* __restrict__ scores, const int32_t* __restrict__ ei, int n, int m,
                                 float threshold, int32_t* parent, uint32_t* err) {
+  pdl_wait();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= m) return;
   const float s = scores[k];
+  int u = ei[k], v = ei[(size_t)m + k];                  // with the score, not after it: one latency
   if (!(s > threshold)) return;
-  int u = ei[k], v = ei[(size_t)m + k];
   if (u < 0 || u >= n || v < 0 || v >= n) return;
   const uint64_t t0 = global_timer_ns();
   for (uint32_t it = 1;; ++it) {
@@ -62,22 +64,13 @@ __global__ void cc_union_kernel(const float* __restrict__ scores, const int32_t*
   }
 }
 
-// Shortens the forest before the final pass: every node points at the root its (path-halving)
-// walk reached.  Racing halving stores can leave some nodes one or more steps below their root,
-// so this pass alone does not give the labels; it only makes the read-only walks short.
-__global__ void cc_compress_kernel(int32_t* parent, int n, uint32_t* err) {
-  const int v = blockIdx.x * blockDim.x + threadIdx.x;
-  if (v >= n) return;
-  const int r = cc_find(parent, v, global_timer_ns());
-  if (r >= 0) parent[v] = r;
-  else atomicOr(err, DEV_ERR_TIMEOUT);
-}
-
-// labels[v] = root of v (the smallest id of its component).  The walk only reads: a path-halving
-// store from another thread could otherwise land on parent[v] after v has written its root and
-// leave v pointing at an intermediate ancestor.  Every value a reader meets is an ancestor (an
-// old parent or a final root), so each walk still ends at its root.
+// labels[v] = root of v.  Every value met on the walk is an ancestor (an old parent or a final root), and
+// the root is the smallest of them.  A walk that gets long halves the path behind it with atomicMin, which
+// can never put back a larger ancestor over a root that another thread has written (a plain store could);
+// the unions' own halving leaves the usual walk too short for that.  A pass of its own that halved paths
+// first cost 7 us of the full event's 29.
 __global__ void cc_flatten_kernel(int32_t* parent, int n, uint32_t* err) {
+  pdl_wait();
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= n) return;
   volatile int32_t* p = parent;
@@ -86,6 +79,10 @@ __global__ void cc_flatten_kernel(int32_t* parent, int n, uint32_t* err) {
   for (uint32_t it = 1;; ++it) {
     const int px = p[x];
     if (px == x) break;
+    if (it > 8) {
+      const int gx = p[px];
+      if (gx < px) atomicMin(parent + x, gx);
+    }
     x = px;
     if ((it & 255u) == 0 && global_timer_ns() - t0 > kUnionLimitNs) {
       atomicOr(err, DEV_ERR_TIMEOUT);

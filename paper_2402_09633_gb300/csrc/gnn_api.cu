@@ -1094,10 +1094,11 @@ int gnn_track_labels(gnn_ctx* ctx, const float* edge_scores, const int32_t* edge
   if (!labels || (n_edges > 0 && (!edge_scores || !edge_index))) return GNN_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const int N = (int)n_nodes, E = (int)n_edges, tb = 256;
-  cc_init_kernel<<<blocks_for(N, tb), tb, 0, st>>>(labels, N);
-  if (E > 0) cc_union_kernel<<<blocks_for(E, tb), tb, 0, st>>>(edge_scores, edge_index, N, E, threshold, labels, ctx->d_err);
-  cc_compress_kernel<<<blocks_for(N, tb), tb, 0, st>>>(labels, N, ctx->d_err);
-  cc_flatten_kernel<<<blocks_for(N, tb), tb, 0, st>>>(labels, N, ctx->d_err);
+  cudaError_t le = launch_pdl(cc_init_kernel, blocks_for(N, tb), tb, 0, st, labels, N);
+  if (le == cudaSuccess && E > 0)
+    le = launch_pdl(cc_union_kernel, blocks_for(E, tb), tb, 0, st, edge_scores, edge_index, N, E, threshold, labels, ctx->d_err);
+  if (le == cudaSuccess) le = launch_pdl(cc_flatten_kernel, blocks_for(N, tb), tb, 0, st, labels, N, ctx->d_err);
+  if (le != cudaSuccess) return cuda_fail(le);
   const cudaError_t err = cudaGetLastError();
   return err == cudaSuccess ? GNN_OK : cuda_fail(err);
 }
