@@ -493,9 +493,9 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
           }
         }
     };
-    auto ld_p = [&](const float* row, int c, float2* t) {      // one row's four pairs
+    auto ld_p = [&](auto keep, const float* row, int c, float2* t) {      // one row's four pairs
       uint32_t m[8];
-      ld_global_32b(row + 32 * c + q8, m);
+      ld_global_32b<decltype(keep)::value>(row + 32 * c + q8, m);
 #pragma unroll
       for (int b = 0; b < 4; ++b) t[b] = make_float2(__uint_as_float(m[2 * b]), __uint_as_float(m[2 * b + 1]));
     };
@@ -529,7 +529,9 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
     };
     // Two T16 state rows -> A operand, AHEAD chunks of loads in flight: whole rows in the two-group kernels
     // (node update 0.170 -> 0.163 ms against three chunks), two chunks where registers are scarcer (edge update
-    // 0.295 -> 0.291).  Rows past the end lie in the buffers' padding to whole tiles.
+    // 0.295 -> 0.291).  The edge kernels read the edge state, and the source's P_s rows, without keeping them in
+    // L1, where the P_d rows of neighbouring edges are read again (0.292 -> 0.287); the node update's own rows
+    // are better kept (0.163, 0.167 streamed).  Rows past the end lie in the buffers' padding to whole tiles.
     auto state_to_a = [&](uint32_t reg, const void* base, int row) {
       constexpr int AHEAD = NCH < 2 * (4 - NG) ? NCH : 2 * (4 - NG);
       using V = typename std::conditional<BF, uint2, float4>::type;
@@ -558,7 +560,10 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
 #pragma unroll
           for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int r = 0; r < 2; ++r) m[c][2 * h + r] = *reinterpret_cast<const V*>(t16(base, row + 8 * r, 2 * c + h));
+            for (int r = 0; r < 2; ++r) {
+              const V* a = reinterpret_cast<const V*>(t16(base, row + 8 * r, 2 * c + h));
+              m[c][2 * h + r] = KIND == TileKind::NodeUpdate ? *a : __ldcs(a);
+            }
       }
     };
     // Runs f(c, t) over the chunks of a region, the next chunk's load in flight meanwhile.
@@ -802,8 +807,8 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
           for (int r = 0; r < 2; ++r) {
             float2 a[4], b[4];
             asm volatile("" : "+r"(ends[r][0]), "+r"(ends[r][1]));   // the row addresses are formed anew, not kept
-            ld_p(p.ps + (size_t)ends[r][0] * H, c, a);
-            ld_p(p.pd + (size_t)ends[r][1] * H, c, b);
+            ld_p(std::false_type{}, p.ps + (size_t)ends[r][0] * H, c, a);
+            ld_p(std::true_type{}, p.pd + (size_t)ends[r][1] * H, c, b);
 #pragma unroll
             for (int k = 0; k < 4; ++k) S[c][2 * k + r] = __fadd2_rn(a[k], b[k]);
           }
