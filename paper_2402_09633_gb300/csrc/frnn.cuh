@@ -162,44 +162,36 @@ __device__ __forceinline__ float frnn_acc(float s, float a, float b) {
   return __fadd_rn(s, __fmul_rn(d, d));
 }
 
-// The pairs of every hit whose chain was kept: the partners' sorted positions, read a chunk at a
-// time, with their hit ids and r gathered together, written oriented from the smaller r.
+// The pairs of every hit whose chain was kept, written oriented from the smaller r: four threads per hit,
+// each a quarter of every chunk's entries (41 -> 26 us on the full event against a thread per hit with
+// fifteen gathers at once; 4 pairs a hit).
+constexpr int kFrnnCopyLanes = 4;
 __global__ void __launch_bounds__(256) frnn_copy_kernel(const float* __restrict__ r_s, int n,
                                                         const int* __restrict__ ids, const int* __restrict__ offsets,
                                                         const int* __restrict__ total, int capacity,
                                                         const int* __restrict__ chunks, int32_t* __restrict__ out) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
+  const int64_t i4 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = (int)(i4 / kFrnnCopyLanes), q = (int)(i4 % kFrnnCopyLanes);
+  if (i4 / kFrnnCopyLanes >= n) return;
   const int n_total = *total;
   if (n_total > capacity || chunks[(size_t)t * kFrnnChunk + kFrnnChunk - 1] == kFrnnLost) return;
-  int pos = offsets[t];
+  const int pos = offsets[t];
   const int cnt = (t + 1 < n ? offsets[t + 1] : n_total) - pos;
   const int i = ids[t];
   const float ri = r_s[t];
   int cur = t;
   for (int base = 0; base < cnt; base += kFrnnChunk - 1) {
-    const int4* c4 = reinterpret_cast<const int4*>(chunks + (size_t)cur * kFrnnChunk);
-    const int4 w0 = c4[0], w1 = c4[1], w2 = c4[2], w3 = c4[3];
-    const int w[kFrnnChunk] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w,
-                               w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
-    const int m = cnt - base;
-    int jj[kFrnnChunk - 1];
-    float rr[kFrnnChunk - 1];
-#pragma unroll
-    for (int k = 0; k < kFrnnChunk - 1; ++k) {
-      jj[k] = k < m ? ids[w[k]] : 0;
-      rr[k] = k < m ? r_s[w[k]] : 0.f;
+    const int* c = chunks + (size_t)cur * kFrnnChunk;
+    const int m = cnt - base < kFrnnChunk - 1 ? cnt - base : kFrnnChunk - 1;
+    for (int k = q; k < m; k += kFrnnCopyLanes) {
+      const int p = c[k];
+      const int jj = ids[p];
+      const float rj = r_s[p];
+      const bool i_first = ri < rj || (ri == rj && i < jj);
+      out[pos + base + k] = i_first ? i : jj;
+      out[(size_t)n_total + pos + base + k] = i_first ? jj : i;
     }
-#pragma unroll
-    for (int k = 0; k < kFrnnChunk - 1; ++k) {
-      if (k < m) {
-        const bool i_first = ri < rr[k] || (ri == rr[k] && i < jj[k]);
-        out[pos] = i_first ? i : jj[k];
-        out[(size_t)n_total + pos] = i_first ? jj[k] : i;
-        ++pos;
-      }
-    }
-    cur = w[kFrnnChunk - 1];
+    if (base + kFrnnChunk - 1 < cnt) cur = c[kFrnnChunk - 1];
   }
 }
 
@@ -217,18 +209,18 @@ __global__ void __launch_bounds__(256) frnn_copy_kernel(const float* __restrict_
 // are 32 for the warp's lanes to test exactly and append to the queries' lists.
 //
 // The bound is the filter's instructions and the latency of its MMAs: on the full event (D = 8, 2.5e9 pairs
-// in the runs, 1.2e6 edges) 22 warp instructions for 128 pairs, two of them MMAs, with 28 warps per SM.  With
+// in the runs, 1.2e6 edges) 22 warp instructions for 128 pairs, two of them MMAs, with 24 warps per SM.  With
 // one thread per hit and the exact test on every candidate the search took 24 fp32 operations a pair, 3.2-4.2
-// ms; with each block's survivors tested on the spot by the lanes that held them 0.86 ms, queued 0.80, and with
-// 72 registers instead of 96 (seven blocks per SM) 0.74.  32 queries per warp test more pairs than they save
-// loads (0.77-0.85).
+// ms; with each block's survivors tested on the spot by the lanes that held them 0.86 ms, queued 0.80, with
+// 72 registers instead of 96 (seven blocks per SM) 0.74, and with the four blocks' loads and MMAs side by
+// side at six blocks per SM 0.72.  32 queries per warp test more pairs than they save loads (0.77-0.85).
 constexpr int kFrnnPairsThreads = 128;
 constexpr int kFrnnQueries = 16;
 constexpr int kFrnnBlockQueries = kFrnnPairsThreads / 32 * kFrnnQueries;
 constexpr int kFrnnQueue = 32 + 8 * kFrnnQueries;                       // below 32 left over, and one block's
 
 template <int CH, int K>
-__global__ void __launch_bounds__(kFrnnPairsThreads, 7) frnn_pairs_kernel(
+__global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     const float4* __restrict__ emb_s, const uint4* __restrict__ frag, const float* __restrict__ r_s, int n, float r2,
     int grid, const int* __restrict__ cell_keys, const int* __restrict__ ids, const int* __restrict__ cell_start,
     int write, int* __restrict__ counts, const int* __restrict__ total, int capacity, int32_t* __restrict__ out,
@@ -440,19 +432,27 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 7) frnn_pairs_kernel(
         for (int b = rp >> 3; b < b1; b += UNROLL) {
           float c[UNROLL][4];
           uint32_t neg = 0u;                       // sign bits
+          uint4 x[UNROLL], y[SETS == 2 ? UNROLL : 1];
 #pragma unroll
           for (int u = 0; u < UNROLL; ++u) {
             const int blk = b + u < b1 ? b + u : b1 - 1;             // past the run's end: its last block again
             const uint4* f = frag + (size_t)blk * (32 * SETS) + lane;
-            const uint4 x = f[0];
-            const float zero[4] = {0.f, 0.f, 0.f, 0.f};
-            mma_m16n8k16(c[u], ah[0][0], ah[0][1], ah[0][0], ah[0][1], x.x, x.y, zero);
-            mma_m16n8k16(c[u], al[0][0], al[0][1], norm[0], norm[1], x.x, x.z, c[u]);
-            if constexpr (SETS == 2) {
-              const uint4 y = f[32];
-              mma_m16n8k16(c[u], ah[1][0], ah[1][1], ah[1][0], ah[1][1], y.x, y.y, c[u]);
-              mma_m16n8k16(c[u], al[1][0], al[1][1], 0u, 0u, y.x, 0u, c[u]);
-            }
+            x[u] = f[0];
+            if constexpr (SETS == 2) y[u] = f[32];
+          }
+          const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int u = 0; u < UNROLL; ++u) mma_m16n8k16(c[u], ah[0][0], ah[0][1], ah[0][0], ah[0][1], x[u].x, x[u].y, zero);
+#pragma unroll
+          for (int u = 0; u < UNROLL; ++u) mma_m16n8k16(c[u], al[0][0], al[0][1], norm[0], norm[1], x[u].x, x[u].z, c[u]);
+          if constexpr (SETS == 2) {
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u) mma_m16n8k16(c[u], ah[1][0], ah[1][1], ah[1][0], ah[1][1], y[u].x, y[u].y, c[u]);
+#pragma unroll
+            for (int u = 0; u < UNROLL; ++u) mma_m16n8k16(c[u], al[1][0], al[1][1], 0u, 0u, y[u].x, 0u, c[u]);
+          }
+#pragma unroll
+          for (int u = 0; u < UNROLL; ++u) {
             neg |= __float_as_uint(c[u][0]) | __float_as_uint(c[u][1]);
             neg |= __float_as_uint(c[u][2]) | __float_as_uint(c[u][3]);
           }

@@ -1057,6 +1057,7 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   const int sb = (int)blocks_for(N, kScanBlock);
   const int pb = (int)blocks_for(N, kFrnnBlockQueries);
   const int fb = (int)blocks_for(blocks_for(N, 8) * (int64_t)32, tb);
+  const int cb = (int)blocks_for((int64_t)N * kFrnnCopyLanes, tb);
   switch (chunks * 8 + K) {
 #define GNN_FRNN_CASE(CH, KK)                                                                                    \
   case CH * 8 + KK:                                                                                              \
@@ -1071,7 +1072,7 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
     frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, frag, r_s, N, r2, grid, kin, vin, cell_start, \
                                                                 1, counts, n_edges, (int)max_edges, edge_index,  \
                                                                 chains, next_chunk, pool, ctx->d_err);           \
-    frnn_copy_kernel<<<nb, tb, 0, st>>>(r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index);      \
+    frnn_copy_kernel<<<cb, tb, 0, st>>>(r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index);      \
     break;
     GNN_FRNN_CASE(1, 3)
     GNN_FRNN_CASE(2, 3)
