@@ -19,8 +19,9 @@
 // and a dependent load each, one block walking every tile's counts.  Here a
 // thread's sixteen elements are loaded at once, a warp ranks its own 512 elements
 // against its own counters without a block barrier, and a warp per digit scans
-// the counts, in seven launches.  1M edges, 300k nodes: 131 -> 66 us, 58 with tiles sorted before they are written; 7,200 edges, 2,000 nodes (one pass):
-// nine launches -> four, 45 us of the tiny event's 164 less.
+// the counts, in seven launches.  1M edges, 300k nodes: 131 -> 66 us, 58 with tiles
+// sorted before they are written; 7,200 edges, 2,000 nodes (one pass): nine launches
+// -> four, 45 us of the tiny event's 164 less.
 #pragma once
 #include <cstdint>
 #include "ptx.cuh"

@@ -10,9 +10,10 @@
 // instead of once per edge.  The node network's first layer on [h, a] is
 // split the same way into W_h and W_a.
 //
-// gnn_infer enqueues: CSR build (validate, radix sort by destination, gather,
-// row pointers) -> node encoder (+ projections) -> edge encoder -> T x (edge
-// update, node update with aggregation + projections) -> classifier.
+// gnn_infer enqueues: CSR build (radix sort by destination, whose first pass
+// validates the endpoints; one kernel gathers the sources and writes the row
+// pointers) -> node encoder (+ projections) -> edge encoder -> T x (edge update,
+// aggregation, node update + projections) -> classifier.
 #include <cuda_runtime.h>
 #include <algorithm>
 #include <atomic>

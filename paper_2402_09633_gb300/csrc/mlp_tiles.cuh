@@ -36,18 +36,17 @@
 //     a ring of stages);
 //   * one worker thread per group warms L2 (bulk prefetch) with the group's next tile.
 //
-// What bounds them (full event, 300k nodes / 1M edges, H = 128, L = 3): the chain of a tile, about 16 us
-// for an edge update (edge state to A 1.3 us, gathers and layer-1 job 2.8, layer-1 epilogue with the last
-// gathers 3.2, two jobs 2.2-2.7 each with their queueing, layer-2 epilogue 2.2, layer 3 and store 1.6),
-// with three chains in flight and a tensor core that is busy half of the time.  Per launch, against two
-// tiles in flight, biases and gammas in the epilogues and first layers on CUDA cores, fp32 / bf16 model:
-// edge update 0.392 -> 0.318 / 0.313 -> 0.237 ms, node update 0.193 -> 0.178 / 0.140 -> 0.125,
-// classifier 0.373 -> 0.297 / 0.331 -> 0.248, edge encoder 0.284 -> 0.222 / 0.219 -> 0.174, node encoder
-// 0.166 -> 0.126 / 0.139 -> 0.101; embedding of 300k hits 0.204 -> 0.079, filter on 1.9M edges
-// 0.90 -> 0.41.  Also measured: one thread per row and four warps per group (every thread then reads
-// every parameter: edge update 0.547 with shared memory, 0.371 through the constant cache); two groups
-// with 104 registers (0.350); gathers of one or three 32-column chunks before the layer-1 wait instead
-// of two (0.328, 0.342).
+// What bounds them (full event, 300k nodes / 1M edges, H = 128, L = 3): the chain of a tile, about 14 us
+// for an edge update (edge state to A, gathers next to the layer-1 job, three epilogues, two more jobs of
+// 0.7-0.8 us with their queueing, store), with three chains in flight and a tensor core that is busy a
+// little over half of the time.  Per launch, against two tiles in flight, biases and gammas in the
+// epilogues and first layers on CUDA cores, fp32 / bf16 model: edge update 0.392 -> 0.288 / 0.313 -> 0.209
+// ms, node update 0.193 -> 0.163 / 0.140 -> 0.118, classifier 0.373 -> 0.262 / 0.331 -> 0.216, edge encoder
+// 0.284 -> 0.192 / 0.219 -> 0.150, node encoder 0.166 -> 0.114 / 0.139 -> 0.101; embedding of 300k hits
+// 0.204 -> 0.078, filter on 1.9M edges 0.90 -> 0.344.  Measured and not taken, in the edge update as it
+// was at 0.32 ms: one thread per row and four warps per group (every thread then reads every parameter:
+// 0.547 with shared memory, 0.371 through the constant cache); two groups with 104 registers (0.350);
+// gathers of one or three 32-column chunks before the layer-1 wait instead of two (0.328, 0.342).
 #pragma once
 #include <climits>
 #include <cstdint>
@@ -79,7 +78,7 @@ __host__ __device__ constexpr bool has_input_job(TileKind k) {
 // Worker groups and threads of a kernel: one warp that issues, and eight per group.
 template <TileKind KIND>
 struct TileRoles {
-    static constexpr int NG = (KIND == TileKind::NodeEncoder || KIND == TileKind::NodeUpdate) ? 2 : 3;
+  static constexpr int NG = (KIND == TileKind::NodeEncoder || KIND == TileKind::NodeUpdate) ? 2 : 3;
   static constexpr int THREADS = 32 + 256 * NG;      // 800 (80 registers each) or 544 (120)
 };
 
