@@ -1,34 +1,69 @@
 // Edge filtering's compaction step: keep the edges whose score is above a
 // threshold, in input order (a stable, deterministic stream compaction).
 //
-// Blocks of 1024 edges: count the kept edges of every block, scan the block
-// counts (one block), then each block writes its kept edges at its offset,
-// ranked in input order (warp ballots within a round of 256 edges, warp totals
-// across a round, a running count across rounds).  The output is the kept edge
-// list [2, n_kept], contiguous (row 1 starts at n_kept), plus the input id of
+// At most kCompactMaxBlocks blocks, each with a run of consecutive edges: one
+// launch counts the kept edges of every block; in the next, each block sums the
+// counts before its own (and all of them: row 1 of the output starts behind row
+// 0) and writes its kept edges there, ranked in input order (warp ballots within
+// 1024 edges, a scan of the 32 ballots' counts, a running count from there on).
+// The output is the kept edge list [2, n_kept], contiguous, plus the input id of
 // every kept edge.
+//
+// The bytes (40 MB for 1.9M edges, half kept) take 6 us; what took the time was latency and launches.
+// A launch of one block that scanned the counts stood between the two, and the scatter went through its
+// 1024 edges in four dependent rounds of load, ballot and two block barriers.  1.9M edges: the filter call
+// 439 -> 432 us (344 of them the MLP); 1,024, 1,216 or 4,096 blocks at most instead of 2,048: 430, 436, 429.
 #pragma once
 #include <cstdint>
+#include "ptx.cuh"
 
 namespace gnn {
 
 constexpr int kCompactThreads = 256;
 constexpr int kCompactRounds = 4;
-constexpr int kCompactBlock = kCompactThreads * kCompactRounds;   // edges per block
+constexpr int kCompactTile = kCompactThreads * kCompactRounds;    // edges a block takes at once
+// More blocks would make the sums over their counts longer (8 loads a thread); fewer leave SMs idle.
+constexpr int kCompactMaxBlocks = 2048;
+
+// Tiles per block, and blocks.
+__host__ __device__ inline int compact_tiles(int64_t m) {
+  const int64_t tiles = (m + kCompactTile - 1) / kCompactTile;
+  return (int)((tiles + kCompactMaxBlocks - 1) / kCompactMaxBlocks);
+}
+inline int compact_blocks(int64_t m) {
+  const int64_t per = (int64_t)compact_tiles(m) * kCompactTile;
+  return (int)((m + per - 1) / per);
+}
 
 __device__ __forceinline__ bool kept(float score, float threshold) { return score > threshold; }  // NaN: no
 
-__global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const float* __restrict__ scores, int m,
-                                                                        float threshold, int* __restrict__ counts) {
-  __shared__ int wsum[kCompactThreads / 32];
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  int c = 0;
+// The calling thread's scores of the tile at `base`: entry r is edge base + r * kCompactThreads + threadIdx.x.
+__device__ __forceinline__ void compact_load(const float* __restrict__ scores, int64_t base, int m, float threshold,
+                                             bool* keep) {
+  float s[kCompactRounds];
 #pragma unroll
   for (int r = 0; r < kCompactRounds; ++r) {
-    const int k = blockIdx.x * kCompactBlock + r * kCompactThreads + t;
-    c += (k < m && kept(scores[k], threshold)) ? 1 : 0;
+    const int64_t k = base + r * kCompactThreads + threadIdx.x;
+    s[r] = k < m ? scores[k] : __int_as_float(0x7fffffff);           // NaN past the end
   }
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+#pragma unroll
+  for (int r = 0; r < kCompactRounds; ++r) keep[r] = kept(s[r], threshold);
+}
+
+__global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const float* __restrict__ scores, int m,
+                                                                        float threshold, int tiles,
+                                                                        int* __restrict__ counts) {
+  __shared__ int wsum[kCompactThreads / 32];
+  pdl_wait();
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  int c = 0;
+  for (int i = 0; i < tiles; ++i) {
+    bool keep[kCompactRounds];
+    compact_load(scores, ((int64_t)blockIdx.x * tiles + i) * kCompactTile, m, threshold, keep);
+#pragma unroll
+    for (int r = 0; r < kCompactRounds; ++r) c += keep[r] ? 1 : 0;
+  }
+  c = __reduce_add_sync(0xffffffffu, c);
   if (lane == 0) wsum[warp] = c;
   __syncthreads();
   if (t == 0) {
@@ -124,34 +159,61 @@ __global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(int* __restrict_
   if (i < n) v[i] = offsets[blockIdx.x] + (warp > 0 ? wsum[warp - 1] : 0) + x - c;
 }
 
+// counts: of gridDim.x blocks, fewer than 2^31 edges in all.  The total goes to *total.
 __global__ void __launch_bounds__(kCompactThreads) compact_scatter_kernel(
-    const float* __restrict__ scores, const int32_t* __restrict__ ei, int m, float threshold,
-    const int* __restrict__ offsets, const int* __restrict__ total, int32_t* __restrict__ out_ei,
+    const float* __restrict__ scores, const int32_t* __restrict__ ei, int m, float threshold, int tiles,
+    const int* __restrict__ counts, int* __restrict__ total, int32_t* __restrict__ out_ei,
     int32_t* __restrict__ out_id) {
-  __shared__ int wcnt[kCompactThreads / 32];
+  constexpr int kWarps = kCompactThreads / 32;
+  static_assert(kWarps * kCompactRounds == 32, "a lane per ballot of a tile");
+  __shared__ int sums[2][kWarps];
+  __shared__ int wcnt[2][32];                            // by round and warp; two tiles' worth in turn
+  pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int n_kept = *total;
-  int run = offsets[blockIdx.x];
-  for (int r = 0; r < kCompactRounds; ++r) {
-    const int k = blockIdx.x * kCompactBlock + r * kCompactThreads + t;
-    const bool keep = k < m && kept(scores[k], threshold);
-    const unsigned ball = __ballot_sync(0xffffffffu, keep);
-    if (lane == 0) wcnt[warp] = __popc(ball);
-    __syncthreads();
-    int before = 0, round_total = 0;
+  int before = 0, all = 0;
+  for (int i = t; i < (int)gridDim.x; i += kCompactThreads) {
+    const int c = counts[i];
+    all += c;
+    before += i < (int)blockIdx.x ? c : 0;
+  }
+  before = __reduce_add_sync(0xffffffffu, before);
+  all = __reduce_add_sync(0xffffffffu, all);
+  if (lane == 0) { sums[0][warp] = before; sums[1][warp] = all; }
+  __syncthreads();
+  int run = 0, n_kept = 0;
 #pragma unroll
-    for (int w = 0; w < kCompactThreads / 32; ++w) {
-      before += w < warp ? wcnt[w] : 0;
-      round_total += wcnt[w];
+  for (int w = 0; w < kWarps; ++w) { run += sums[0][w]; n_kept += sums[1][w]; }
+  if (blockIdx.x == 0 && t == 0) *total = n_kept;
+  for (int i = 0; i < tiles; ++i) {
+    const int64_t base = ((int64_t)blockIdx.x * tiles + i) * kCompactTile;
+    bool keep[kCompactRounds];
+    unsigned ball[kCompactRounds];
+    compact_load(scores, base, m, threshold, keep);
+    int u[kCompactRounds], v[kCompactRounds];
+#pragma unroll
+    for (int r = 0; r < kCompactRounds; ++r) {
+      ball[r] = __ballot_sync(0xffffffffu, keep[r]);
+      if (lane == 0) wcnt[i & 1][r * kWarps + warp] = __popc(ball[r]);
+      const int64_t k = base + r * kCompactThreads + t;
+      if (keep[r]) { u[r] = ei[k]; v[r] = ei[(size_t)m + k]; }
     }
-    if (keep) {
-      const int pos = run + before + __popc(ball & ((1u << lane) - 1u));
-      out_ei[pos] = ei[k];
-      out_ei[(size_t)n_kept + pos] = ei[(size_t)m + k];
-      if (out_id) out_id[pos] = k;
-    }
-    run += round_total;
     __syncthreads();
+    const int own = wcnt[i & 1][lane];
+    int x = own;                                         // inclusive scan over (round, warp)
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+#pragma unroll
+    for (int r = 0; r < kCompactRounds; ++r) {
+      const int first = __shfl_sync(0xffffffffu, x - own, r * kWarps + warp);
+      if (!keep[r]) continue;
+      const int pos = run + first + __popc(ball[r] & ((1u << lane) - 1u));
+      out_ei[pos] = u[r];
+      out_ei[(size_t)n_kept + pos] = v[r];
+      if (out_id) out_id[pos] = (int)(base + r * kCompactThreads + t);
+    }
+    run += __shfl_sync(0xffffffffu, x, 31);
   }
 }
 

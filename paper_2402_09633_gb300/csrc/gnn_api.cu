@@ -890,13 +890,15 @@ int gnn_filter_edges(gnn_ctx* ctx, const float* node_feats, const int32_t* edge_
     if (bf) launch_tile<TileKind::Filter, 64, true>(ctx, ctx->filter_plan, p, st);
     else launch_tile<TileKind::Filter, 64, false>(ctx, ctx->filter_plan, p, st);
   }
-  const int nb = (int)blocks_for(E, kCompactBlock);
+  const int tiles = compact_tiles(E), nb = compact_blocks(E);
   int* counts = ctx->keys_a;
-  compact_count_kernel<<<nb, kCompactThreads, 0, st>>>(edge_scores, E, threshold, counts);
-  compact_scan_kernel<<<1, 1024, 0, st>>>(counts, nb, n_kept);
-  compact_scatter_kernel<<<nb, kCompactThreads, 0, st>>>(edge_scores, edge_index, E, threshold, counts, n_kept,
-                                                          kept_index, kept_id);
-  const cudaError_t err = cudaGetLastError();
+  cudaError_t err = launch_pdl(compact_count_kernel, nb, kCompactThreads, 0, st, (const float*)edge_scores, E, threshold,
+                               tiles, counts);
+  if (err == cudaSuccess)
+    err = launch_pdl(compact_scatter_kernel, nb, kCompactThreads, 0, st, (const float*)edge_scores, edge_index, E,
+                     threshold, tiles, (const int*)counts, n_kept, kept_index, kept_id);
+  if (err != cudaSuccess) return cuda_fail(err);
+  err = cudaGetLastError();
   return err == cudaSuccess ? GNN_OK : cuda_fail(err);
 }
 
