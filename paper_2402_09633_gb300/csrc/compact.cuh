@@ -73,54 +73,17 @@ __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const fl
   }
 }
 
-// Exclusive scan of the block counts in place (one block of 1024 threads); the total goes to *total.
-// The sums are taken in 64 bits and the total saturates at INT32_MAX, so a caller that compares the
-// total with its capacity (below INT32_MAX) sees an overflow as "too many" (offsets past the
-// overflow point are then meaningless and must not be used).
-__global__ void __launch_bounds__(1024) compact_scan_kernel(int* __restrict__ counts, int n_blocks,
-                                                            int* __restrict__ total) {
-  __shared__ long long wsum[32];
-  __shared__ long long carry;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  if (t == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n_blocks; base += 1024) {
-    const int i = base + t;
-    const long long v = i < n_blocks ? counts[i] : 0;
-    long long x = v;                                       // inclusive scan inside the warp
-    for (int o = 1; o < 32; o <<= 1) {
-      const long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (lane == 31) wsum[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-      long long w = wsum[lane];
-      for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(0xffffffffu, w, o);
-        if (lane >= o) w += y;
-      }
-      wsum[lane] = w;                                      // inclusive over warps
-    }
-    __syncthreads();
-    const long long excl = carry + (warp > 0 ? wsum[warp - 1] : 0) + x - v;
-    if (i < n_blocks) counts[i] = (int)excl;
-    __syncthreads();
-    if (t == 0) carry += wsum[31];
-    __syncthreads();
-  }
-  if (t == 0) *total = carry > 0x7fffffffLL ? 0x7fffffff : (int)carry;
-}
-
-// Exclusive scan of a long int array in place, in three launches: scan_reduce_kernel (sum of
-// every 1024 entries, saturated at INT32_MAX), compact_scan_kernel over those sums (offsets and
-// the total), scan_apply_kernel (offset plus the scan inside each 1024 entries).  A total above
-// INT32_MAX saturates there; the offsets are then meaningless and the caller must not use them.
+// Exclusive scan of a long int array in place, in two launches: scan_reduce_kernel (sum of every 1024
+// entries, saturated at INT32_MAX), scan_apply_kernel (each block sums the sums before its own, and scans
+// its 1024 entries from there; the total of all goes to *total).  Sums are taken in 64 bits and the total
+// saturates at INT32_MAX, so a caller that compares it with its capacity (below INT32_MAX) sees an
+// overflow as "too many"; the offsets are then meaningless and must not be used.
 constexpr int kScanBlock = 1024;
 
 __global__ void __launch_bounds__(kScanBlock) scan_reduce_kernel(const int* __restrict__ v, int n,
                                                                  int* __restrict__ sums) {
   __shared__ long long wsum[32];
+  pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int i = blockIdx.x * kScanBlock + t;
   long long x = i < n ? v[i] : 0;
@@ -135,28 +98,51 @@ __global__ void __launch_bounds__(kScanBlock) scan_reduce_kernel(const int* __re
 }
 
 __global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(int* __restrict__ v, int n,
-                                                                const int* __restrict__ offsets) {
+                                                                const int* __restrict__ sums,
+                                                                int* __restrict__ total) {
+  __shared__ long long part[2][32];
   __shared__ int wsum[32];
+  pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int i = blockIdx.x * kScanBlock + t;
   const int c = i < n ? v[i] : 0;
+  long long before = 0, all = 0;
+  for (int b = t; b < (int)gridDim.x; b += kScanBlock) {
+    const long long s = sums[b];
+    all += s;
+    before += b < (int)blockIdx.x ? s : 0;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    before += __shfl_xor_sync(0xffffffffu, before, o);
+    all += __shfl_xor_sync(0xffffffffu, all, o);
+  }
   int x = c;
   for (int o = 1; o < 32; o <<= 1) {
     const int y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
+  if (lane == 0) { part[0][warp] = before; part[1][warp] = all; }
   if (lane == 31) wsum[warp] = x;
   __syncthreads();
   if (warp == 0) {
     int w = wsum[lane];
+    long long b = part[0][lane], a = part[1][lane];
+    for (int o = 16; o > 0; o >>= 1) {
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+    }
     for (int o = 1; o < 32; o <<= 1) {
       const int y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    wsum[lane] = w;
+    wsum[lane] = (int)b + w;                             // offset of the next warp's first entry
+    if (lane == 0) {
+      part[0][0] = b;
+      if (blockIdx.x == 0) *total = a > 0x7fffffffLL ? 0x7fffffff : (int)a;
+    }
   }
   __syncthreads();
-  if (i < n) v[i] = offsets[blockIdx.x] + (warp > 0 ? wsum[warp - 1] : 0) + x - c;
+  if (i < n) v[i] = (warp > 0 ? wsum[warp - 1] : (int)part[0][0]) + x - c;
 }
 
 // counts: of gridDim.x blocks, fewer than 2^31 edges in all.  The total goes to *total.

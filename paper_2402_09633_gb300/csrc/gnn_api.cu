@@ -1042,40 +1042,34 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   int* hist = block_sums + nb;
   int* cell_start = hist + radix_hist_ints(N);
   int* next_chunk = cell_start + n_cells + 1;
-  if (K == 4) frnn_cell_kernel<4><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, cells);
-  else frnn_cell_kernel<3><<<nb, tb, 0, st>>>(embedding, N, emb_dim, grid, cells);
+  cudaError_t le = cudaSuccess;                           // first launch error
+  auto chk = [&](cudaError_t e) { if (le == cudaSuccess) le = e; };
+  if (K == 4) chk(launch_pdl(frnn_cell_kernel<4>, nb, tb, 0, st, embedding, N, emb_dim, grid, cells, next_chunk));
+  else chk(launch_pdl(frnn_cell_kernel<3>, nb, tb, 0, st, embedding, N, emb_dim, grid, cells, next_chunk));
   int* const skeys[2] = {keys_a, keys_b};
   int* const svals[2] = {vals_a, vals_b};
-  cudaError_t serr = cudaSuccess;
-  const int sorted = launch_radix_sort(RadixKeys{cells}, N, n_cells - 1, skeys, svals, hist, st, &serr);
-  if (serr != cudaSuccess) return cuda_fail(serr);
+  const int sorted = launch_radix_sort(RadixKeys{cells}, N, n_cells - 1, skeys, svals, hist, st, &le);
+  if (le != cudaSuccess) return cuda_fail(le);
   const int *kin = skeys[sorted], *vin = svals[sorted];
-  csr_rowptr_kernel<<<blocks_for((int64_t)n_cells + 1, tb), tb, 0, st>>>(kin, N, n_cells, cell_start);
-  {
-    const cudaError_t e0 = cudaMemsetAsync(next_chunk, 0, sizeof(int), st);
-    if (e0 != cudaSuccess) return cuda_fail(e0);
-  }
   const float r2 = radius * radius;
   const int xs = ctx->cfg.n_node_feat;
   const int sb = (int)blocks_for(N, kScanBlock);
   const int pb = (int)blocks_for(N, kFrnnBlockQueries);
   const int fb = (int)blocks_for(blocks_for(N, 8) * (int64_t)32, tb);
   const int cb = (int)blocks_for((int64_t)N * kFrnnCopyLanes, tb);
+  const int sc = (int)blocks_for((int64_t)n_cells + 1, tb);
   switch (chunks * 8 + K) {
 #define GNN_FRNN_CASE(CH, KK)                                                                                    \
   case CH * 8 + KK:                                                                                              \
-    frnn_gather_kernel<CH><<<nb, tb, 0, st>>>(embedding, node_feats, xs, N, emb_dim, vin, emb_s, r_s);         \
-    frnn_fragments_kernel<CH><<<fb, tb, 0, st>>>(emb_s, N, frag);                                                \
-    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, frag, r_s, N, r2, grid, kin, vin, cell_start, \
-                                                                0, counts, nullptr, 0, nullptr, chains,          \
-                                                                next_chunk, pool, ctx->d_err);                   \
-    scan_reduce_kernel<<<sb, kScanBlock, 0, st>>>(counts, N, block_sums);                                      \
-    compact_scan_kernel<<<1, 1024, 0, st>>>(block_sums, sb, n_edges);                                            \
-    scan_apply_kernel<<<sb, kScanBlock, 0, st>>>(counts, N, block_sums);                                       \
-    frnn_pairs_kernel<CH, KK><<<pb, kFrnnPairsThreads, 0, st>>>(emb_s, frag, r_s, N, r2, grid, kin, vin, cell_start, \
-                                                                1, counts, n_edges, (int)max_edges, edge_index,  \
-                                                                chains, next_chunk, pool, ctx->d_err);           \
-    frnn_copy_kernel<<<cb, tb, 0, st>>>(r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index);      \
+    chk(launch_pdl(frnn_layout_kernel<CH>, fb + sc, tb, 0, st, embedding, node_feats, xs, N, emb_dim, vin, kin, n_cells,\
+                   fb, (float2*)emb_s, r_s, frag, cell_start));                                                        \
+    chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \
+                   cell_start, 0, counts, nullptr, 0, nullptr, chains, next_chunk, pool, ctx->d_err));                 \
+    chk(launch_pdl(scan_reduce_kernel, sb, kScanBlock, 0, st, counts, N, block_sums));                                 \
+    chk(launch_pdl(scan_apply_kernel, sb, kScanBlock, 0, st, counts, N, block_sums, n_edges));                         \
+    chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \
+                   cell_start, 1, counts, n_edges, (int)max_edges, edge_index, chains, next_chunk, pool, ctx->d_err)); \
+    chk(launch_pdl(frnn_copy_kernel, cb, tb, 0, st, r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index));\
     break;
     GNN_FRNN_CASE(1, 3)
     GNN_FRNN_CASE(2, 3)
@@ -1087,6 +1081,7 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
     GNN_FRNN_CASE(4, 4)
 #undef GNN_FRNN_CASE
   }
+  if (le != cudaSuccess) return cuda_fail(le);
   const cudaError_t err = cudaGetLastError();
   return err == cudaSuccess ? GNN_OK : cuda_fail(err);
 }
