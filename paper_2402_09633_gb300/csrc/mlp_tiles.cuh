@@ -38,8 +38,8 @@
 //
 // What bounds them (full event, 300k nodes / 1M edges, H = 128, L = 3): the chain of a tile, about 14 us
 // for an edge update (edge state to A, gathers next to the layer-1 job, three epilogues, two more jobs of
-// 0.7-0.8 us with their queueing, store), with three chains in flight and a tensor core that is busy a
-// little over half of the time.  Per launch, against two tiles in flight, biases and gammas in the
+// 0.7-0.8 us with their queueing, store), with three chains in flight: tensor pipe 47 % active, DRAM
+// 54 %, issue 32 %.  Per launch, against two tiles in flight, biases and gammas in the
 // epilogues and first layers on CUDA cores, fp32 / bf16 model: edge update 0.392 -> 0.288 / 0.313 -> 0.209
 // ms, node update 0.193 -> 0.163 / 0.140 -> 0.118, classifier 0.373 -> 0.262 / 0.331 -> 0.216, edge encoder
 // 0.284 -> 0.192 / 0.219 -> 0.150, node encoder 0.166 -> 0.114 / 0.139 -> 0.101; embedding of 300k hits
@@ -351,7 +351,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
         const uint32_t acc0 = (p.job_acc[j] || bias) ? 1u : 0u;
         const uint64_t ones = sdesc_kmajor_plain(smem_u32(consts));
         const uint64_t bdesc = sdesc_kmajor_plain(smem_u32(consts) + G::ONES_BYTES + (bias ? bias - 1 : 0) * G::BIAS_BYTES);
-        // covers for groups without a tile this round, at the streamed weights' stage
+        // covers for groups without a tile in the last round, at the streamed weights' stage
         const int covers = (!resident && g == 0 && i_g[0] + NG > n_my) ? i_g[0] + NG - n_my : 0;
         tc_fence_after();
         if (elect_one()) {
