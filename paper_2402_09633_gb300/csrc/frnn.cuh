@@ -296,6 +296,8 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     const unsigned peers = __match_any_sync(FULL, hit ? qi : kFrnnQueries);       // this query's partners
     const int rank = __popc(peers & below), cnt = __popc(peers), leader = __ffs(peers) - 1;
     const int had = hit ? w.found[qi] : 0, at = had + rank;
+    int cur = 0;                                   // counting pass: the chunk being filled
+    bool gone = false;
     if (write) {
       if (hit) {
         const int i = ids[t0 + qi], jj = ids[pf];
@@ -308,8 +310,8 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
       constexpr int C = kFrnnChunk - 1;            // entries per chunk
       const int have = had > 0 ? (had - 1) / C : 0;                               // chunks filled or begun, less one
       const int more = hit ? (had + cnt - 1) / C - have : 0;                      // chunks this batch begins
-      const int cur = hit ? w.cur[qi] : 0;
-      const bool gone = hit && w.lost[qi];
+      cur = hit ? w.cur[qi] : 0;
+      gone = hit && w.lost[qi];
       int base = 0;
       if (hit && rank == 0 && more > 0 && !gone) {
         base = atomicAdd(next_chunk, more);
@@ -325,13 +327,17 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
         const int k = at / C - have;               // 0: the chunk being filled
         chunks[(size_t)(k == 0 ? cur : n + base + k - 1) * kFrnnChunk + at % C] = pf;
       }
-      if (hit && rank == 0) {
-        if (keep && more > 0) w.cur[qi] = n + base + more - 1;
-        if (base < 0) w.lost[qi] = 1;
+      if (keep && more > 0) cur = n + base + more - 1;
+      gone = gone || base < 0;
+    }
+    __syncwarp();                                  // every lane has read found, cur and lost
+    if (hit && rank == 0) {
+      w.found[qi] = had + cnt;
+      if (!write) {
+        w.cur[qi] = cur;
+        w.lost[qi] = gone;
       }
     }
-    __syncwarp();                                  // every lane has read found and cur
-    if (hit && rank == 0) w.found[qi] = had + cnt;
     __syncwarp();
   };
 

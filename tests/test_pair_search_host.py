@@ -1,0 +1,104 @@
+"""The pair search's kernels (csrc/frnn.cuh), run on the CPU from their own source: no data race in a
+warp's shared memory, and the edge list of the oracle for chains of several chunks, used-up pools, and
+pairs at the radius for every set of operands and row level."""
+import ctypes
+import re
+
+import numpy as np
+import pytest
+
+from oracle import gnn_oracle as O
+from tests import host_cuda
+
+MAIN = r"""
+#include "ptx.cuh"
+#include "frnn.cuh"
+using namespace gnn;
+template <int CH, int K>
+static void build(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap, int32_t* out,
+                  int* n_edges, uint32_t* err) {
+  const int grid = frnn_grid(radius, K);
+  int n_cells = 1;
+  for (int k = 0; k < K; ++k) n_cells *= grid;
+  std::vector<int> cells(n), ids(n), keys(n), starts(n_cells + 1), counts(n), chains((size_t)(n + pool) * kFrnnChunk, -99);
+  std::vector<float4> emb_s((size_t)n * CH);
+  std::vector<float> r_s(n);
+  std::vector<uint4> frag((size_t)(n + 7) / 8 * 32 * ((CH + 1) / 2));
+  int next = -1;
+  const int nb = (n + 255) / 256;
+  host::launch(nb, 256, [&] { frnn_cell_kernel<K>(emb, n, dim, grid, cells.data(), &next); });
+  for (int i = 0; i < n; ++i) ids[i] = i;
+  std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) { return cells[a] < cells[b]; });
+  for (int i = 0; i < n; ++i) keys[i] = cells[ids[i]];
+  const int fb = ((n + 7) / 8 * 32 + 255) / 256;
+  host::launch(fb, 256, [&] {
+    frnn_layout_kernel<CH>(emb, x, 1, n, dim, ids.data(), keys.data(), n_cells, fb, (float2*)emb_s.data(), r_s.data(),
+                           frag.data(), starts.data());
+  });
+  for (int j = 0; j <= n_cells; ++j) starts[j] = std::lower_bound(keys.begin(), keys.end(), j) - keys.begin();
+  auto pairs = [&](int write) {
+    host::launch((n + kFrnnBlockQueries - 1) / kFrnnBlockQueries, kFrnnPairsThreads, [&] {
+      frnn_pairs_kernel<CH, K>(emb_s.data(), frag.data(), r_s.data(), n, radius * radius, grid, keys.data(), ids.data(),
+                               starts.data(), write, counts.data(), n_edges, cap, out, chains.data(), &next, pool, err);
+    });
+  };
+  pairs(0);
+  int sum = 0;
+  for (int& c : counts) { const int k = c; c = sum; sum += k; }
+  *n_edges = sum;
+  pairs(1);
+  host::launch((4 * n + 255) / 256, 256, [&] {
+    frnn_copy_kernel(r_s.data(), n, ids.data(), counts.data(), n_edges, cap, chains.data(), out);
+  });
+}
+extern "C" int build_graph(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap,
+                           int32_t* out, int* n_edges) {
+  uint32_t err = 0;
+  host::races = 0;
+  if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
+  else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
+  else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
+  else build<4, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
+  return err ? -1 : host::races;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    text = host_cuda.source("frnn.cuh")
+    shared = host_cuda.between(text, "  struct Warp {", "  };")
+    checked = re.sub(r"\b(int|unsigned char) (?=\w+\[)", r"host::Cell<\1> ", shared)
+    assert checked.count("host::Cell") == 5
+    return host_cuda.compile_host(tmp_path_factory.mktemp("host"), MAIN, [("frnn.cuh", text.replace(shared, checked))])
+
+
+def build(lib, emb, r, radius, pool=None):
+    n, dim = emb.shape
+    pool = n if pool is None else pool
+    cap = n * n
+    out = np.full(2 * cap, -1, np.int32)
+    m = ctypes.c_int(0)
+    p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
+    races = lib.build_graph(p(emb), p(r), n, dim, ctypes.c_float(radius), pool, cap, p(out), ctypes.byref(m))
+    return out[:2 * m.value].reshape(2, -1), races
+
+
+def ordered(ei):
+    e = ei.T.astype(np.int64)
+    return e[np.lexsort((e[:, 1], e[:, 0]))]
+
+
+@pytest.mark.parametrize("pool", [None, 0, 7])
+def test_chains_of_several_chunks(lib, pool):
+    """Clumps of up to 60 hits within the radius of each other: a batch of 32 pairs holds several partners of
+    one query, whose chain begins new chunks in the middle of it."""
+    rng = np.random.default_rng(3)
+    centres = rng.standard_normal((4, 8))
+    emb = np.repeat(centres / np.linalg.norm(centres, axis=1, keepdims=True), [60, 33, 16, 1], axis=0)
+    emb = (emb + 0.001 * rng.standard_normal(emb.shape)).astype(np.float32)[rng.permutation(110)]
+    r = rng.random(110).astype(np.float32)
+    ei, races = build(lib, emb, r, 0.1, pool)
+    np.testing.assert_array_equal(ordered(ei), O.radius_graph(emb, r, 0.1))
+    np.testing.assert_array_equal(ei, build(lib, emb, r, 0.1)[0])     # the pool changes nothing
+    assert races == 0, f"{races} unordered accesses to shared memory"
