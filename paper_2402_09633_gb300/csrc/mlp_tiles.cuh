@@ -414,15 +414,21 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
         }
       }
     }
-    // before teardown (and the TMEM release), the last MMAs of each group have completed
+    // Before teardown (and the TMEM release), every commit has arrived, not only the one of the same MMAs that
+    // the workers wait for: an arrival after the block's exit could meet the next block's shared memory ...
 #pragma unroll
     for (int g = 0; g < NG; ++g)
       if (seq_g[g] > 0) drain_wait(&d_full[g], (seq_g[g] - 1) & 1);
-    // ... and every weight copy has landed (the last one per stage)
+    if constexpr (NG == 3)
+      for (uint32_t k = 0; k < (uint32_t)NSPARE; ++k)
+        if (const uint32_t uses = sp_uses + (k < sp ? 1u : 0u)) drain_wait(&spare_free[k], (uses - 1) & 1);
+    // ... and so has every weight copy (the last one per stage, and the release of its stage)
     drain_wait(c_full, 0);
     if (resident) drain_wait(&w_full[0], 0);
-    for (uint32_t k = loaded > (uint32_t)STAGES ? loaded - STAGES : 0u; k < loaded; ++k)
+    for (uint32_t k = loaded > (uint32_t)STAGES ? loaded - STAGES : 0u; k < loaded; ++k) {
       drain_wait(&w_full[k % STAGES], (k / STAGES) & 1);
+      drain_wait(&w_empty[k % STAGES], (k / STAGES) & 1);
+    }
     __syncwarp();
   } else {
     // Worker groups: eight warps to a group, sixteen rows of its tile to a warp (half of a tensor-memory
