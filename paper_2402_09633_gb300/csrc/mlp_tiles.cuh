@@ -677,10 +677,13 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
     [[maybe_unused]] float2 x_in[8];
     [[maybe_unused]] int ends[2][2];           // rows' endpoints: source, destination
     [[maybe_unused]] int valid = 0, valid_next = 0;   // filter: bit r, endpoints of row r in range
+    // This thread's row r of tile t, in arithmetic that wraps: rows of a tile past the end, which the loads
+    // below are asked for and leave out, may not fit an int.
+    auto tile_row = [&](int t, int r) { return (int)((uint32_t)t * kTileRows + (uint32_t)(trow + 8 * r)); };
     auto load_ends = [&](int t) {              // endpoints of this thread's two edges of tile t
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
-        const int k = t * kTileRows + trow + 8 * r;
+        const int k = tile_row(t, r);
         const bool in = t < p.n_tiles && k < p.n_rows;
         if constexpr (KIND == TileKind::Filter) {
           ends[r][0] = in ? p.ei_in[k] : -1;
@@ -708,7 +711,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
           xs = p.x + (size_t)ends[r][0] * p.x_stride;
           xd = p.x + (size_t)ends[r][1] * p.x_stride;
         } else {
-          const int k = t * kTileRows + trow + 8 * r;
+          const int k = tile_row(t, r);
           xs = xd = p.x + (size_t)(t < p.n_tiles && k < p.n_rows ? k : 0) * p.x_stride;
         }
         if constexpr (KIND == TileKind::EdgeEncoder) {       // columns 0 and 1 of both ends; (dr, dphi) at use
