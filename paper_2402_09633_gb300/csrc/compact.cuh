@@ -73,20 +73,27 @@ __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const fl
   }
 }
 
-// Exclusive scan of a long int array in place, in two launches: scan_reduce_kernel (sum of every 1024
-// entries, saturated at INT32_MAX), scan_apply_kernel (each block sums the sums before its own, and scans
-// its 1024 entries from there; the total of all goes to *total).  Sums are taken in 64 bits and the total
-// saturates at INT32_MAX, so a caller that compares it with its capacity (below INT32_MAX) sees an
-// overflow as "too many"; the offsets are then meaningless and must not be used.
+// Exclusive scan of a long int array in place, in two launches of compact_blocks(n) blocks, each with a run of
+// `tiles` = compact_tiles(n) times 1024 consecutive entries: scan_reduce_kernel (sum of every block's entries,
+// saturated at INT32_MAX), scan_apply_kernel (each block sums the sums before its own, and scans its entries
+// from there; the total of all goes to *total).  At most 2,048 blocks, so that their sums over the block sums
+// stay behind the entries themselves: with 1,024 entries a block whatever n, they grew with its square.
+// Sums are taken in 64 bits and the total saturates at INT32_MAX, so a caller that compares it with its
+// capacity (below INT32_MAX) sees an overflow as "too many"; the offsets are then meaningless and must not
+// be used.
 constexpr int kScanBlock = 1024;
+static_assert(kScanBlock == kCompactTile, "compact_tiles and compact_blocks count in entries of a scan block");
 
-__global__ void __launch_bounds__(kScanBlock) scan_reduce_kernel(const int* __restrict__ v, int n,
+__global__ void __launch_bounds__(kScanBlock) scan_reduce_kernel(const int* __restrict__ v, int n, int tiles,
                                                                  int* __restrict__ sums) {
   __shared__ long long wsum[32];
   pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int i = blockIdx.x * kScanBlock + t;
-  long long x = i < n ? v[i] : 0;
+  long long x = 0;
+  for (int k = 0; k < tiles; ++k) {
+    const int64_t i = ((int64_t)blockIdx.x * tiles + k) * kScanBlock + t;
+    x += i < n ? v[i] : 0;
+  }
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   if (lane == 0) wsum[warp] = x;
   __syncthreads();
@@ -97,15 +104,13 @@ __global__ void __launch_bounds__(kScanBlock) scan_reduce_kernel(const int* __re
   }
 }
 
-__global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(int* __restrict__ v, int n,
+__global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(int* __restrict__ v, int n, int tiles,
                                                                 const int* __restrict__ sums,
                                                                 int* __restrict__ total) {
   __shared__ long long part[2][32];
-  __shared__ int wsum[32];
+  __shared__ int wsum[2][32];                            // two tiles' worth in turn
   pdl_wait();
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int i = blockIdx.x * kScanBlock + t;
-  const int c = i < n ? v[i] : 0;
   long long before = 0, all = 0;
   for (int b = t; b < (int)gridDim.x; b += kScanBlock) {
     const long long s = sums[b];
@@ -116,33 +121,36 @@ __global__ void __launch_bounds__(kScanBlock) scan_apply_kernel(int* __restrict_
     before += __shfl_xor_sync(0xffffffffu, before, o);
     all += __shfl_xor_sync(0xffffffffu, all, o);
   }
-  int x = c;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
   if (lane == 0) { part[0][warp] = before; part[1][warp] = all; }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  if (warp == 0) {
-    int w = wsum[lane];
-    long long b = part[0][lane], a = part[1][lane];
-    for (int o = 16; o > 0; o >>= 1) {
-      b += __shfl_xor_sync(0xffffffffu, b, o);
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-    }
+  unsigned run = 0;                                      // offset of the tile's first entry (meaningless past 2^31)
+  for (int k = 0; k < tiles; ++k) {
+    const int64_t i = ((int64_t)blockIdx.x * tiles + k) * kScanBlock + t;
+    const int c = i < n ? v[i] : 0;
+    unsigned x = (unsigned)c;
     for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, w, o);
+      const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[k & 1][warp] = (int)x;
+    __syncthreads();
+    if (k == 0) {
+      long long b = part[0][lane], a = part[1][lane];
+      for (int o = 16; o > 0; o >>= 1) {
+        b += __shfl_xor_sync(0xffffffffu, b, o);
+        a += __shfl_xor_sync(0xffffffffu, a, o);
+      }
+      run = (unsigned)b;
+      if (blockIdx.x == 0 && t == 0) *total = a > 0x7fffffffLL ? 0x7fffffff : (int)a;
+    }
+    unsigned w = (unsigned)wsum[k & 1][lane];            // inclusive scan over the warps' sums
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
-    wsum[lane] = (int)b + w;                             // offset of the next warp's first entry
-    if (lane == 0) {
-      part[0][0] = b;
-      if (blockIdx.x == 0) *total = a > 0x7fffffffLL ? 0x7fffffff : (int)a;
-    }
+    const unsigned first = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+    if (i < n) v[i] = (int)(run + (warp > 0 ? first : 0u) + x - (unsigned)c);
+    run += __shfl_sync(0xffffffffu, w, 31);
   }
-  __syncthreads();
-  if (i < n) v[i] = (warp > 0 ? wsum[warp - 1] : (int)part[0][0]) + x - c;
 }
 
 // counts: of gridDim.x blocks, fewer than 2^31 edges in all.  The total goes to *total.

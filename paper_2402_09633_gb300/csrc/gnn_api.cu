@@ -1053,7 +1053,7 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   const int *kin = skeys[sorted], *vin = svals[sorted];
   const float r2 = radius * radius;
   const int xs = ctx->cfg.n_node_feat;
-  const int sb = (int)blocks_for(N, kScanBlock);
+  const int sb = compact_blocks(N), scan_tiles = compact_tiles(N);
   const int pb = (int)blocks_for(N, kFrnnBlockQueries);
   const int fb = (int)blocks_for(blocks_for(N, 8) * (int64_t)32, tb);
   const int cb = (int)blocks_for((int64_t)N * kFrnnCopyLanes, tb);
@@ -1065,8 +1065,8 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
                    fb, (float2*)emb_s, r_s, frag, cell_start));                                                        \
     chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \
                    cell_start, 0, counts, nullptr, 0, nullptr, chains, next_chunk, pool, ctx->d_err));                 \
-    chk(launch_pdl(scan_reduce_kernel, sb, kScanBlock, 0, st, counts, N, block_sums));                                 \
-    chk(launch_pdl(scan_apply_kernel, sb, kScanBlock, 0, st, counts, N, block_sums, n_edges));                         \
+    chk(launch_pdl(scan_reduce_kernel, sb, kScanBlock, 0, st, counts, N, scan_tiles, block_sums));                     \
+    chk(launch_pdl(scan_apply_kernel, sb, kScanBlock, 0, st, counts, N, scan_tiles, block_sums, n_edges));             \
     chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \
                    cell_start, 1, counts, n_edges, (int)max_edges, edge_index, chains, next_chunk, pool, ctx->d_err)); \
     chk(launch_pdl(frnn_copy_kernel, cb, tb, 0, st, r_s, N, vin, counts, n_edges, (int)max_edges, chains, edge_index));\

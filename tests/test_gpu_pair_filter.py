@@ -103,3 +103,20 @@ def test_values_off_the_sphere(dim):
         want = O.radius_graph(emb, r, 1.0)
     assert want.shape[0] > 100
     np.testing.assert_array_equal(_edges(emb, r, 1.0, 250000), want)
+
+
+@pytest.mark.gpu
+def test_more_hits_than_one_scan_tile_per_block():
+    """Above 2,048 x 1,024 hits a block of the counts' scan takes two tiles: a lattice of isolated hits, 200,000
+    of which have one partner."""
+    rng = np.random.default_rng(1)
+    n, m = 2_000_003, 200_000
+    at = rng.permutation(40 ** 4)[:n]
+    emb = np.stack([at // 40 ** k % 40 for k in range(4)], 1) * (1.8 / 39) - 0.9
+    owner = rng.permutation(n)[:m]
+    emb = np.concatenate([emb, emb[owner] + [0, 0, 0, 0.01]]).astype(np.float32)
+    r = rng.random(n + m).astype(np.float32)
+    pair = np.stack([owner, n + np.arange(m)], 1)
+    first = (r[pair[:, 0]] < r[pair[:, 1]]) | ((r[pair[:, 0]] == r[pair[:, 1]]) & (pair[:, 0] < pair[:, 1]))
+    pair = np.where(first[:, None], pair, pair[:, ::-1])
+    np.testing.assert_array_equal(_edges(emb, r, 0.02, 1 << 20), pair[np.lexsort((pair[:, 1], pair[:, 0]))])
