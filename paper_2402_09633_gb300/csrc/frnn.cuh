@@ -343,6 +343,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
 
   // A fragments of queries g and g + 8: rows r = 0, 1
   uint32_t ah[SETS][2], al[SETS][2], an[2];
+  bool tame = true;                                // no query is wild
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     const int t = t0 + g + 8 * r < n ? t0 + g + 8 * r : n - 1;
@@ -357,6 +358,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     na += __shfl_xor_sync(FULL, na, 1);
     na += __shfl_xor_sync(FULL, na, 2);
     const bool wild = !(na < kFrnnWildNorm);
+    tame = tame && !wild;
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
       if (wild) v[s] = make_float2(0.f, 0.f);
@@ -404,11 +406,18 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     p1 = cell_start[row * d1 + hi];
   };
   int level = 0, d0 = 1;
-  const int fine = groups_at(grid);
-  if (fine > 2) {
-    // A coarser level costs its MMAs, found from its first row's runs; level 0 about 120 MMAs' time per
-    // row of cells (63 rows looked up, a few runs of four MMAs and their set-up).  Taken when it is cheaper,
-    // the finest first.  With level 0 throughout, 2,000 hits took 187 us and 30,000 took 234.
+  const int cells = __shfl_sync(FULL, key, 31 - __clz(wanted)) - __shfl_sync(FULL, key, __ffs(wanted) - 1);
+  if (cells >= 2 && __all_sync(FULL, tame)) {      // (a wild query has every candidate tested: the fewest, then)
+    // Two or more cells from the first query to the last.  A coarser level costs its blocks, by the first row's
+    // runs; level 0 the time of about eight blocks (of one set of operands) for each run it looks up, however few
+    // candidates that has.  Taken when it is cheaper, the finest first.  Builds of unit vectors with half of that
+    // for a run, no notice of the sets and only where queries lay in three rows or more -> as it is: 2M hits D = 4
+    // 2.04 -> 1.38 ms, D = 6 at small radius 2.20 -> 1.24; 300,000 hits D = 6 380 -> 289 us, D = 12 at small radius
+    // 484 -> 328; 30,000 hits D = 8 234 -> 144 us; full event (queries in one cell) 0.74 ms both.  Half as much
+    // again for a run: 300,000 hits D = 6 at large radius 574 -> 593 us, 2M 2.21 -> 2.35 ms.
+    int runs0 = 1;
+    for (int k = 1; k < K; ++k) runs0 *= W;
+    const long long fine = 8LL * ((runs0 + 1) / 2) * groups_at(grid);
     for (int v = 1, e0 = grid; v < K; ++v, e0 *= grid) {
       const int e1 = e0 * grid, gs = groups_at(e1);
       const int first = __ffs(wanted) - 1;
@@ -416,7 +425,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
       int p, p1;
       row_run(v, e0, e1, first, 31 - __clz(same), lane, p, p1);
       const int blocks = p < p1 ? (p1 - p) / 8 + 6 : 0;
-      if ((long long)gs * (__reduce_add_sync(FULL, blocks) + 40) < 120LL * fine) {
+      if ((long long)gs * (SETS * __reduce_add_sync(FULL, blocks) + 40) < fine) {
         level = v;
         d0 = e0;
         break;

@@ -48,7 +48,7 @@ static std::vector<Warp> warps;
 static std::vector<char> stacks;
 static ucontext_t scheduler;
 static std::function<void()> body;
-static int current, races, epochs;                     // epochs: begun so far, by any warp
+static int current, races, mmas, epochs;               // mmas: of a lane; epochs: begun so far, by any warp
 constexpr size_t kStack = 64 * 1024;
 
 inline void die(const char* why) { std::fprintf(stderr, "host_cuda: %s\n", why); std::abort(); }
@@ -186,6 +186,7 @@ inline unsigned __ballot_sync(unsigned, int p) {
   return b;
 }
 inline int __any_sync(unsigned m, int p) { return __ballot_sync(m, p) != 0; }
+inline int __all_sync(unsigned m, int p) { return __ballot_sync(m, p) == m; }
 inline unsigned __match_any_sync(unsigned, int x) {
   const host::Word10* w = host_collect("__match_any_sync", x);
   unsigned b = 0;
@@ -223,6 +224,7 @@ inline float __bfloat162float(__nv_bfloat16 x) { return __uint_as_float((uint32_
 inline void host_mma(float* d, uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1,
                      const float* c) {
   const int lane = host_lane(), g = lane >> 2, q = lane & 3;
+  host::mmas += lane == 0;
   const float c0[4] = {c[0], c[1], c[2], c[3]};
   const host::Word10* w = host::all_lanes("mma", {{a0, a1, a2, a3, b0, b1}});
   auto half = [](uint32_t x, int h) { return __uint_as_float(h ? x & 0xffff0000u : x << 16); };

@@ -54,13 +54,14 @@ static void build(const float* emb, const float* x, int n, int dim, float radius
 extern "C" int build_graph(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap,
                            int32_t* out, int* n_edges) {
   uint32_t err = 0;
-  host::races = 0;
+  host::races = host::mmas = 0;
   if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else build<4, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   return err ? -1 : host::races;
 }
+extern "C" int mmas() { return host::mmas; }
 """
 
 
@@ -102,3 +103,21 @@ def test_chains_of_several_chunks(lib, pool):
     np.testing.assert_array_equal(ordered(ei), O.radius_graph(emb, r, 0.1))
     np.testing.assert_array_equal(ei, build(lib, emb, r, 0.1)[0])     # the pool changes nothing
     assert races == 0, f"{races} unordered accesses to shared memory"
+
+
+@pytest.mark.parametrize("dim", [4, 12])
+def test_sparse_hits_share_runs(lib, dim):
+    """Parallel lines of hits, one every other cell of a row: a row's own 63 runs would take a batch of four blocks
+    for a few candidates each; a coarser level takes half of the blocks."""
+    rng = np.random.default_rng(0)
+    line = np.stack(np.meshgrid(*[np.arange(5)] * 3, indexing="ij"), -1).reshape(-1, 3) * (2 / 64) + 0.01
+    emb = np.zeros((line.shape[0], 20, dim))
+    emb[:, :, :3] = line[:, None]
+    emb[:, :, 3] = (np.arange(20) * 2 - 20) * (2 / 64) + 0.01
+    emb = (emb.reshape(-1, dim) + 1e-4 * rng.random((2500, 1))).astype(np.float32)
+    r = rng.random(2500).astype(np.float32)
+    ei, _ = build(lib, emb, r, 0.02)
+    np.testing.assert_array_equal(ordered(ei), O.radius_graph(emb, r, 0.02))
+    warps, mma = (2500 + 15) // 16, 2 if dim <= 8 else 4
+    blocks = lib.mmas() / warps / mma                # of eight candidates, per sixteen hits
+    assert blocks <= 120, f"{blocks:.0f} blocks (one row of cells at a time: 178)"
