@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
       }
       hit = s < r2;
     }
+    if (!__any_sync(FULL, hit)) return;            // usual where the radius is below the filter's resolution
     const unsigned peers = __match_any_sync(FULL, hit ? qi : kFrnnQueries);       // this query's partners
     const int rank = __popc(peers & below), cnt = __popc(peers), leader = __ffs(peers) - 1;
     const int had = hit ? w.found[qi] : 0, at = had + rank;

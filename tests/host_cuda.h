@@ -48,7 +48,7 @@ static std::vector<Warp> warps;
 static std::vector<char> stacks;
 static ucontext_t scheduler;
 static std::function<void()> body;
-static int current, races, mmas, epochs;               // mmas: of a lane; epochs: begun so far, by any warp
+static int current, races, mmas, matches, epochs;      // mmas, matches: by any warp; epochs: begun so far
 constexpr size_t kStack = 64 * 1024;
 
 inline void die(const char* why) { std::fprintf(stderr, "host_cuda: %s\n", why); std::abort(); }
@@ -188,6 +188,7 @@ inline unsigned __ballot_sync(unsigned, int p) {
 inline int __any_sync(unsigned m, int p) { return __ballot_sync(m, p) != 0; }
 inline int __all_sync(unsigned m, int p) { return __ballot_sync(m, p) == m; }
 inline unsigned __match_any_sync(unsigned, int x) {
+  host::matches += host_lane() == 0;
   const host::Word10* w = host_collect("__match_any_sync", x);
   unsigned b = 0;
   for (int i = 0; i < 32; ++i) b |= (w[i].v[0] == (uint32_t)x ? 1u : 0u) << i;

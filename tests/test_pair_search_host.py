@@ -54,7 +54,7 @@ static void build(const float* emb, const float* x, int n, int dim, float radius
 extern "C" int build_graph(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap,
                            int32_t* out, int* n_edges) {
   uint32_t err = 0;
-  host::races = host::mmas = 0;
+  host::races = host::mmas = host::matches = 0;
   if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
@@ -62,6 +62,7 @@ extern "C" int build_graph(const float* emb, const float* x, int n, int dim, flo
   return err ? -1 : host::races;
 }
 extern "C" int mmas() { return host::mmas; }
+extern "C" int matches() { return host::matches; }
 """
 
 
@@ -121,3 +122,15 @@ def test_sparse_hits_share_runs(lib, dim):
     warps, mma = (2500 + 15) // 16, 2 if dim <= 8 else 4
     blocks = lib.mmas() / warps / mma                # of eight candidates, per sixteen hits
     assert blocks <= 120, f"{blocks:.0f} blocks (one row of cells at a time: 178)"
+
+
+def test_pairs_below_the_filters_resolution(lib):
+    """Hits 0.002 apart, searched at half of that: the filter lets all of them through (it is right to about 0.01 on
+    unit vectors), the exact test none, and no lists are gone through for them."""
+    emb = np.zeros((200, 8), np.float32)
+    emb[:, 0] = 0.6
+    emb[:, 4] = 0.4 + 0.002 * (np.arange(200) % 20)
+    emb[:, 5] = 0.4 + 0.002 * (np.arange(200) // 20)
+    ei, races = build(lib, emb, np.zeros(200, np.float32), 0.001)
+    assert ei.shape[1] == 0 and races == 0
+    assert lib.matches() == 0
