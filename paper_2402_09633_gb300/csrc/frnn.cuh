@@ -76,9 +76,10 @@ __global__ void frnn_cell_kernel(const float* __restrict__ emb, int n, int dim, 
 //   f = (1 - c)(|a|^2 + |b|^2) - 2 (ah bh + ah bl + al bh) - r2',  c = 2^-14, r2' slightly above r2.
 // Against the squared distance d the parts left out, the splits' rounding and the accumulation are off
 // by less than 3e-5 (|a|^2 + |b|^2) / 2 + 1e-5 (|a|^2 + |b|^2), under half of c (|a|^2 + |b|^2): a pair
-// with d < r2 never gives f >= 0.  Only pairs with f < 0 are tested exactly.  A hit that is not finite
-// or whose squared norm passes 1e18 is "wild": its operands are zero and its norm slot -1e30, so that f
-// is finite everywhere and such a hit is tested exactly against every candidate.
+// with d < r2 never gives f >= 0.  Only pairs with f < 0 are tested exactly.  A hit whose squared norm
+// passes 1e18 is "wild": its operands are zero and its norm slot -1e30, so that f is finite everywhere and
+// such a hit is tested exactly against every candidate.  A hit with an infinite or NaN coordinate is within
+// no radius of any (its differences are infinite or NaN): its norm slot is one that no radius reaches.
 // K slots: 0-7 -2ah.bh, 8-15 -2ah.bl, 16-23 -2al.bh, 24-26 |a|^2 parts x 1, 27-29 1 x |b|^2 parts.
 constexpr float kFrnnSlack = 1.0f / 16384.0f;
 constexpr float kFrnnWildNorm = 1e18f, kFrnnWild = -1e30f;
@@ -94,6 +95,16 @@ __device__ __forceinline__ void frnn_parts(float v, float* q) {
     q[k] = __bfloat162float(__float2bfloat16_rn(v));
     v -= q[k];
   }
+}
+
+// Whether any coordinate of this quad's hit is infinite or NaN (each lane holds some of them; called by whole warps).
+template <int SETS>
+__device__ __forceinline__ bool frnn_odd(const float2* v) {
+  float z = 0.f;
+#pragma unroll
+  for (int s = 0; s < SETS; ++s) z += (v[s].x - v[s].x) + (v[s].y - v[s].y);         // 0 or NaN
+  const unsigned odd = __ballot_sync(0xffffffffu, !(z == 0.f));
+  return ((odd >> (threadIdx.x & 28)) & 15u) != 0u;
 }
 
 // What the search reads, from the sorted order, in one launch.  Blocks below frag_blocks: sorted copies
@@ -144,8 +155,8 @@ __global__ void frnn_layout_kernel(const float* __restrict__ emb, const float* _
   }
   nb += __shfl_xor_sync(0xffffffffu, nb, 1);
   nb += __shfl_xor_sync(0xffffffffu, nb, 2);
-  const bool wild = !(nb < kFrnnWildNorm);
-  nb = pos >= n ? -kFrnnWild : wild ? kFrnnWild : nb * (1.0f - kFrnnSlack);
+  const bool wild = !(nb < kFrnnWildNorm), odd = frnn_odd<SETS>(v);
+  nb = pos >= n || odd ? -kFrnnWild : wild ? kFrnnWild : nb * (1.0f - kFrnnSlack);
   float q[3];
   frnn_parts(nb, q);
 #pragma unroll
@@ -358,7 +369,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     }
     na += __shfl_xor_sync(FULL, na, 1);
     na += __shfl_xor_sync(FULL, na, 2);
-    const bool wild = !(na < kFrnnWildNorm);
+    const bool wild = !(na < kFrnnWildNorm), odd = frnn_odd<SETS>(v);
     tame = tame && !wild;
 #pragma unroll
     for (int s = 0; s < SETS; ++s) {
@@ -368,7 +379,7 @@ __global__ void __launch_bounds__(kFrnnPairsThreads, 6) frnn_pairs_kernel(
     }
     const float reach = fminf(r2 * (1.0f + 1.0f / 4096.0f) + 1e-35f, 1e29f);
     float u[3];
-    frnn_parts(wild ? kFrnnWild : na * (1.0f - kFrnnSlack) - reach, u);
+    frnn_parts(odd ? -kFrnnWild : wild ? kFrnnWild : na * (1.0f - kFrnnSlack) - reach, u);
     an[r] = q == 0 ? pack_bf16x2(u[0], u[1]) : q == 1 ? pack_bf16x2(u[2], 1.f) : q == 2 ? pack_bf16x2(1.f, 1.f) : 0u;
   }
 

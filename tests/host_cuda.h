@@ -48,7 +48,7 @@ static std::vector<Warp> warps;
 static std::vector<char> stacks;
 static ucontext_t scheduler;
 static std::function<void()> body;
-static int current, races, mmas, matches, epochs;      // mmas, matches: by any warp; epochs: begun so far
+static int current, races, mmas, matches, tests, epochs;   // mmas, matches: by any warp; epochs: begun so far
 constexpr size_t kStack = 64 * 1024;
 
 inline void die(const char* why) { std::fprintf(stderr, "host_cuda: %s\n", why); std::abort(); }

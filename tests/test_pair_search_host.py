@@ -54,7 +54,7 @@ static void build(const float* emb, const float* x, int n, int dim, float radius
 extern "C" int build_graph(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap,
                            int32_t* out, int* n_edges) {
   uint32_t err = 0;
-  host::races = host::mmas = host::matches = 0;
+  host::races = host::mmas = host::matches = host::tests = 0;
   if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
   else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
@@ -63,6 +63,7 @@ extern "C" int build_graph(const float* emb, const float* x, int n, int dim, flo
 }
 extern "C" int mmas() { return host::mmas; }
 extern "C" int matches() { return host::matches; }
+extern "C" int tests() { return host::tests; }
 """
 
 
@@ -72,7 +73,8 @@ def lib(tmp_path_factory):
     shared = host_cuda.between(text, "  struct Warp {", "  };")
     checked = re.sub(r"\b(int|unsigned char) (?=\w+\[)", r"host::Cell<\1> ", shared)
     assert checked.count("host::Cell") == 5
-    return host_cuda.compile_host(tmp_path_factory.mktemp("host"), MAIN, [("frnn.cuh", text.replace(shared, checked))])
+    text = host_cuda.replace(text.replace(shared, checked), "      hit = s < r2;", "      hit = s < r2; ++host::tests;")
+    return host_cuda.compile_host(tmp_path_factory.mktemp("host"), MAIN, [("frnn.cuh", text)])
 
 
 def build(lib, emb, r, radius, pool=None):
@@ -134,3 +136,20 @@ def test_pairs_below_the_filters_resolution(lib):
     ei, races = build(lib, emb, np.zeros(200, np.float32), 0.001)
     assert ei.shape[1] == 0 and races == 0
     assert lib.matches() == 0
+
+
+def test_infinite_and_nan_hits_are_no_candidates(lib):
+    """A hit with an infinite or NaN coordinate is within no radius of any: no exact test for it.  Long hits
+    whose squares overflow are still tested."""
+    rng = np.random.default_rng(1)
+    emb = rng.standard_normal((120, 8)).astype(np.float32)
+    emb[::3, 2] = np.nan
+    emb[1::6, 7] = np.inf
+    emb[2::12] = np.float32(1e20)
+    emb[5] = -np.inf
+    r = rng.random(120).astype(np.float32)
+    ei, _ = build(lib, emb, r, 3.0)
+    with np.errstate(invalid="ignore", over="ignore"):
+        np.testing.assert_array_equal(ordered(ei), O.radius_graph(emb, r, 3.0))
+    ei, _ = build(lib, np.full((200, 8), np.nan, np.float32), np.zeros(200, np.float32), 0.2)
+    assert ei.shape[1] == 0 and lib.tests() == 0
