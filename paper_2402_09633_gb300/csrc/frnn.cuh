@@ -20,11 +20,12 @@
 // The test is the full squared distance, summed over the coordinates in order
 // with one rounding per product and per sum (no fused multiply-add; the zero
 // padding adds exact zeros), against radius^2 rounded to fp32; a tensor-core
-// filter that never turns a pair down decides which pairs it is made for.  Each
-// pair becomes one edge, oriented from the hit with the smaller r (column 0 of the
-// node features, hit id as tie-break).  A counting pass, an exclusive scan of
-// the per-hit counts and a writing pass make the output order deterministic: by
-// the visiting hit's sorted position, then by row and position of the partner.
+// filter that never turns a pair down decides which pairs it is made for (many
+// hits in up to three dimensions do without it).  Each pair becomes one edge,
+// oriented from the hit with the smaller r (column 0 of the node features, hit
+// id as tie-break).  A counting pass, an exclusive scan of the per-hit counts and
+// a writing pass make the output order deterministic: by the visiting hit's
+// sorted position, then by row and position of the partner.
 // The counting pass also keeps the partners it finds, in the order it finds
 // them, in a chain of 64-byte chunks per hit (its own first chunk, further ones
 // from a pool), so the writing pass copies instead of searching again; a hit
@@ -216,6 +217,63 @@ __global__ void __launch_bounds__(256) frnn_copy_kernel(const float* __restrict_
     }
     if (base + kFrnnChunk - 1 < cnt) cur = c[kFrnnChunk - 1];
   }
+}
+
+// The counting pass of many hits in at most three dimensions, a thread per hit: the runs of its own five cells in
+// the 13 rows, every candidate tested exactly, partners kept as frnn_pairs_kernel keeps them (whose writing pass
+// takes the hits that lost their chains).  An exact test is twelve operations there, and the filter of
+// frnn_pairs_kernel lets much of what it sees through (it is right to about 0.01 between unit vectors, in cells of
+// 1/64), so it only pays while threads are too few to fill the GPU.  Builds with the filter / by single hits: 2M
+// hits D = 2 33.0 / 14.6 ms, D = 3 1.60 / 1.11; 300,000 hits D = 2 1.08 / 0.63; 100,000 hits D = 1 420 / 251 us,
+// D = 2 257 / 199, D = 3 102 / 97; 65,000 hits 244 / 190, 163 / 154, 91 / 91; 16,000 hits D = 3 76 / 80.
+// Above three dimensions the filter is ahead on unit vectors at every size (10M hits D = 4 10.2 ms, by single hits,
+// with a slower sort, 12.9).  It is behind where hits fill the cube [-1, 1]^4, which an embedding's do not (2M hits
+// with 10 edges each 1.81 ms, 1.46; one hit to two cells, no edges, 10M 8.4, 6.4).
+constexpr int kFrnnSingleThreads = 128;
+constexpr int kFrnnSingleHits = 65536;
+__global__ void __launch_bounds__(kFrnnSingleThreads) frnn_single_kernel(
+    const float4* __restrict__ emb_s, int n, float r2, int grid, const int* __restrict__ cell_keys,
+    const int* __restrict__ cell_start, int* __restrict__ counts, int* __restrict__ chunks, int* __restrict__ next_chunk,
+    int max_extra) {
+  constexpr int C = kFrnnChunk - 1;                // entries per chunk
+  pdl_wait();
+  const int t = blockIdx.x * kFrnnSingleThreads + threadIdx.x;
+  if (t >= n) return;
+  const float4 x = emb_s[t];
+  const int key = cell_keys[t], c2 = key % grid, c1 = key / grid % grid, c0 = key / grid / grid;
+  const int lo = c2 < kFrnnReach ? 0 : c2 - kFrnnReach, hi = c2 + kFrnnReach >= grid ? grid : c2 + kFrnnReach + 1;
+  int found = 0, cur = t, fill = 0;
+  bool lost = false;
+  chunks[(size_t)t * kFrnnChunk + C] = -1;         // link of the first chunk: none yet
+  for (int a = 0; a <= kFrnnReach && c0 + a < grid; ++a)
+    for (int b = a == 0 ? 0 : -kFrnnReach; b <= kFrnnReach; ++b) {
+      if (c1 + b < 0 || c1 + b >= grid) continue;
+      const int row = ((c0 + a) * grid + c1 + b) * grid, p1 = cell_start[row + hi];
+      // 32 candidates at a time, so that the loop over them is free of the rare partner's work
+      for (int p = a == 0 && b == 0 ? t + 1 : cell_start[row + lo]; p < p1; p += 32) {
+        const int m = p1 - p < 32 ? p1 - p : 32;
+        uint32_t hits = 0u;
+        for (int k = 0; k < m; ++k) {
+          const float4 y = emb_s[p + k];
+          hits |= (frnn_acc(frnn_acc(frnn_acc(0.f, x.x, y.x), x.y, y.y), x.z, y.z) < r2 ? 1u : 0u) << k;
+        }
+        for (; hits; hits &= hits - 1) {
+          if (fill == C && !lost) {
+            const int next = atomicAdd(next_chunk, 1);
+            lost = next < 0 || next >= max_extra;
+            if (!lost) {
+              chunks[(size_t)cur * kFrnnChunk + C] = n + next;
+              cur = n + next;
+              fill = 0;
+            }
+          }
+          if (!lost) chunks[(size_t)cur * kFrnnChunk + fill++] = p + __ffs(hits) - 1;
+          ++found;
+        }
+      }
+    }
+  counts[t] = found;
+  if (lost) chunks[(size_t)t * kFrnnChunk + C] = kFrnnLost;
 }
 
 // A warp searches for sixteen consecutive sorted positions t (its queries).  write == 0: counts[t] =

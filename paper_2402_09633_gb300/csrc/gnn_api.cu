@@ -1063,8 +1063,12 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   case CH * 8 + KK:                                                                                              \
     chk(launch_pdl(frnn_layout_kernel<CH>, fb + sc, tb, 0, st, embedding, node_feats, xs, N, emb_dim, vin, kin, n_cells,\
                    fb, (float2*)emb_s, r_s, frag, cell_start));                                                        \
-    chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \
-                   cell_start, 0, counts, nullptr, 0, nullptr, chains, next_chunk, pool, ctx->d_err));                 \
+    if (KK == 3 && N >= kFrnnSingleHits)                                                                               \
+      chk(launch_pdl(frnn_single_kernel, blocks_for(N, kFrnnSingleThreads), kFrnnSingleThreads, 0, st, emb_s, N, r2,   \
+                     grid, kin, cell_start, counts, chains, next_chunk, pool));                                        \
+    else                                                                                                               \
+      chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin, \
+                     cell_start, 0, counts, nullptr, 0, nullptr, chains, next_chunk, pool, ctx->d_err));               \
     chk(launch_pdl(scan_reduce_kernel, sb, kScanBlock, 0, st, counts, N, scan_tiles, block_sums));                     \
     chk(launch_pdl(scan_apply_kernel, sb, kScanBlock, 0, st, counts, N, scan_tiles, block_sums, n_edges));             \
     chk(launch_pdl(frnn_pairs_kernel<CH, KK>, pb, kFrnnPairsThreads, 0, st, emb_s, frag, r_s, N, r2, grid, kin, vin,   \

@@ -106,6 +106,38 @@ def test_values_off_the_sphere(dim):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dim,radius", [(1, 2e-5), (2, 0.006), (3, 0.04)])
+@pytest.mark.parametrize("n", [65535, 65536, 70001])
+def test_single_hits_in_few_dimensions(n, dim, radius):
+    """Both sides of the hit count from which up to three dimensions are searched by single hits; byte for byte the
+    same with chunks for few and for none of the hits with more than 15 partners."""
+    import ctypes
+    import torch
+    from paper_2402_09633_gb300 import InteractionNetwork
+    kd = pytest.importorskip("scipy.spatial")
+    rng = np.random.default_rng(n + dim)
+    emb = rng.uniform(-1, 1, (n, dim)).astype(np.float32)
+    emb[:200] = emb[0] + np.float32(radius / 5) * rng.standard_normal((200, dim)).astype(np.float32)
+    emb[200] = np.nan
+    x = np.zeros((n, 3), np.float32)
+    x[:, 0] = rng.random(n)
+    cfg = S.ModelConfig(3, 2, 64, 0, 2)
+    net = InteractionNetwork(cfg, S.pack_blob(cfg, S.init_weights(cfg, 0)))
+    net.lib.gnn_debug_graph_pool.argtypes = [ctypes.c_void_p, ctypes.c_int64]
+    lists = []
+    for pool in (-1, 0, 100):
+        net.lib.gnn_debug_graph_pool(net.handle, pool)
+        lists.append(net.build_graph(torch.from_numpy(emb).cuda(), torch.from_numpy(x).cuda(), radius, 20 * n)[0].cpu().numpy())
+    net.close()
+    assert all(a.tobytes() == lists[0].tobytes() for a in lists)
+    ok = np.delete(np.arange(n), 200)
+    cand = kd.cKDTree(emb[ok].astype(np.float64)).query_pairs(radius * 1.001, output_type="ndarray")
+    want = O.radius_graph(emb, x[:, 0], radius, np.sort(ok[cand], 1))
+    got = lists[0].T.astype(np.int64)
+    np.testing.assert_array_equal(got[np.lexsort((got[:, 1], got[:, 0]))], want)
+
+
+@pytest.mark.gpu
 def test_more_hits_than_one_scan_tile_per_block():
     """Above 2,048 x 1,024 hits a block of the counts' scan takes two tiles: a lattice of isolated hits, 200,000
     of which have one partner."""

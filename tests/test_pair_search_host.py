@@ -16,7 +16,7 @@ MAIN = r"""
 using namespace gnn;
 template <int CH, int K>
 static void build(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap, int32_t* out,
-                  int* n_edges, uint32_t* err) {
+                  int* n_edges, uint32_t* err, bool single) {
   const int grid = frnn_grid(radius, K);
   int n_cells = 1;
   for (int k = 0; k < K; ++k) n_cells *= grid;
@@ -42,7 +42,13 @@ static void build(const float* emb, const float* x, int n, int dim, float radius
                                starts.data(), write, counts.data(), n_edges, cap, out, chains.data(), &next, pool, err);
     });
   };
-  pairs(0);
+  if (K == 3 && single)
+    host::launch((n + kFrnnSingleThreads - 1) / kFrnnSingleThreads, kFrnnSingleThreads, [&] {
+      frnn_single_kernel(emb_s.data(), n, radius * radius, grid, keys.data(), starts.data(), counts.data(), chains.data(),
+                         &next, pool);
+    });
+  else
+    pairs(0);
   int sum = 0;
   for (int& c : counts) { const int k = c; c = sum; sum += k; }
   *n_edges = sum;
@@ -52,13 +58,13 @@ static void build(const float* emb, const float* x, int n, int dim, float radius
   });
 }
 extern "C" int build_graph(const float* emb, const float* x, int n, int dim, float radius, int pool, int cap,
-                           int32_t* out, int* n_edges) {
+                           int32_t* out, int* n_edges, int single) {
   uint32_t err = 0;
   host::races = host::mmas = host::matches = host::tests = 0;
-  if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
-  else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
-  else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
-  else build<4, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err);
+  if (dim < 4) build<1, 3>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err, single);
+  else if (dim <= 8) build<2, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err, single);
+  else if (dim <= 12) build<3, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err, single);
+  else build<4, 4>(emb, x, n, dim, radius, pool, cap, out, n_edges, &err, single);
   return err ? -1 : host::races;
 }
 extern "C" int mmas() { return host::mmas; }
@@ -77,14 +83,14 @@ def lib(tmp_path_factory):
     return host_cuda.compile_host(tmp_path_factory.mktemp("host"), MAIN, [("frnn.cuh", text)])
 
 
-def build(lib, emb, r, radius, pool=None):
+def build(lib, emb, r, radius, pool=None, single=False):
     n, dim = emb.shape
     pool = n if pool is None else pool
     cap = n * n
     out = np.full(2 * cap, -1, np.int32)
     m = ctypes.c_int(0)
     p = lambda a: a.ctypes.data_as(ctypes.c_void_p)  # noqa: E731
-    races = lib.build_graph(p(emb), p(r), n, dim, ctypes.c_float(radius), pool, cap, p(out), ctypes.byref(m))
+    races = lib.build_graph(p(emb), p(r), n, dim, ctypes.c_float(radius), pool, cap, p(out), ctypes.byref(m), int(single))
     return out[:2 * m.value].reshape(2, -1), races
 
 
@@ -153,3 +159,16 @@ def test_infinite_and_nan_hits_are_no_candidates(lib):
         np.testing.assert_array_equal(ordered(ei), O.radius_graph(emb, r, 3.0))
     ei, _ = build(lib, np.full((200, 8), np.nan, np.float32), np.zeros(200, np.float32), 0.2)
     assert ei.shape[1] == 0 and lib.tests() == 0
+
+
+@pytest.mark.parametrize("dim", [1, 2, 3])
+def test_single_hits_and_filter_agree(lib, dim):
+    """The counting pass by single hits gives the lists of the filter's, with room for the chains and without."""
+    rng = np.random.default_rng(dim)
+    emb = rng.uniform(-1, 1, (300, dim)).astype(np.float32)
+    emb[:120] = emb[0] + 0.02 * rng.standard_normal((120, dim)).astype(np.float32)     # runs and chains of several parts
+    r = rng.random(300).astype(np.float32)
+    want, _ = build(lib, emb, r, 0.05)
+    np.testing.assert_array_equal(ordered(want), O.radius_graph(emb, r, 0.05))
+    for pool in (None, 0, 40):
+        np.testing.assert_array_equal(build(lib, emb, r, 0.05, pool, single=True)[0], want)
