@@ -166,10 +166,11 @@ int gnn_infer_host(gnn_ctx* ctx, const float* node_feats, const int32_t* edge_in
  *   n_edges    device int32 [1], output: the number of edges found
  * When n_edges exceeds max_edges nothing is written to edge_index, *n_edges still holds the
  * count (saturated at INT32_MAX), and gnn_status reports GNN_ERR_CAPACITY: call again with room
- * for that many.  The order
- * of the edges is deterministic.  Uses a scratch buffer of the context (grown on demand,
- * synchronous then): besides the sorted copies, 128 bytes per hit for the partner chains the
- * counting pass keeps (see gnn_debug_graph_pool) and 64 (128 for emb_dim > 8) for the pair filter.  Errors: INVALID_ARG (radius <= 0, emb_dim out
+ * for that many.  The order of the edges is deterministic.  Uses a scratch buffer of the context
+ * (grown on demand, synchronous then): besides the sorted copies, 128 bytes per hit for the partner
+ * chains the counting pass keeps (see gnn_debug_graph_pool) and 64 (128 for emb_dim > 8) for the
+ * pair filter; half of the former suffice, with a second search for hits with more than 15 partners,
+ * and are made do with where memory does not hold all.  Errors: INVALID_ARG (radius <= 0, emb_dim out
  * of range, null pointer, bad sizes), OOM, CUDA.
  */
 int gnn_embed_load(gnn_ctx* ctx, const void* weights_host, size_t weights_bytes);

@@ -82,6 +82,7 @@ struct gnn_ctx {
   float embed_eps = 0.f;
   int* aux = nullptr;
   size_t aux_ints = 0;
+  bool aux_tight = false;              // the scratch was made without the default pool of partner chunks
   int64_t graph_pool = -1;             // graph building: pool chunks for partner chains (-1: one per hit)
   uint32_t* d_err = nullptr;
   // workspace
@@ -1012,22 +1013,36 @@ int gnn_build_graph(gnn_ctx* ctx, const float* embedding, int emb_dim, const flo
   // partner chains kept by the counting pass: one first chunk per hit, pool chunks after them (a hit
   // whose chain cannot grow is searched again by the writing pass)
   const int64_t pool64 = ctx->graph_pool >= 0 ? ctx->graph_pool : (int64_t)N;
-  const int pool = (int)(pool64 < (int64_t)INT_MAX - N ? pool64 : (int64_t)INT_MAX - N);
+  int pool = (int)(pool64 < (int64_t)INT_MAX - N ? pool64 : (int64_t)INT_MAX - N);
   // scratch: emb_s [N, 4 * chunks] (first, 16-byte aligned), partner chunks, r_s, keys/vals (two
   // buffers each), per-hit counts, per-block sums, radix histograms, cell starts, the pool counter
   const int nb = (int)blocks_for(N, tb);
-  const size_t chain_ints = ((size_t)N + (size_t)pool) * kFrnnChunk;
   // B fragments of the pair filter: 16 bytes x 32 lanes per eight hits and set of eight coordinates
   const int sets = (chunks + 1) / 2;
   const size_t frag_ints = ((size_t)N + 7) / 8 * 128 * (size_t)sets;
-  const size_t need = 4 * (size_t)chunks * N + frag_ints + chain_ints + 6 * (size_t)N + (size_t)nb + radix_hist_ints(N) +
-                      (size_t)n_cells + 2;
+  const size_t fixed = 4 * (size_t)chunks * N + frag_ints + (size_t)N * kFrnnChunk + 6 * (size_t)N + (size_t)nb +
+                       radix_hist_ints(N) + (size_t)n_cells + 2;
+  // Where memory does not hold the default pool, the build goes on without one: the same edges, found twice
+  // for hits with more than 15 partners.  A scratch made so (aux_tight) is kept for calls that it can serve.
+  if (ctx->aux_tight && ctx->graph_pool < 0 && fixed <= ctx->aux_ints)
+    pool = (int)std::min<size_t>(pool, (ctx->aux_ints - fixed) / kFrnnChunk);
+  const size_t need = fixed + (size_t)pool * kFrnnChunk;
   if (need > ctx->aux_ints) {
     if (ctx->aux) { cudaStreamSynchronize(st); cudaFree(ctx->aux); ctx->aux = nullptr; ctx->aux_ints = 0; }
-    const cudaError_t err = dev_alloc((void**)&ctx->aux, need * sizeof(int));
+    ctx->aux_tight = false;
+    size_t ints = need;
+    cudaError_t err = dev_alloc((void**)&ctx->aux, ints * sizeof(int));
+    if (err == cudaErrorMemoryAllocation && ctx->graph_pool < 0) {
+      (void)cudaGetLastError();
+      ctx->aux_tight = true;
+      pool = 0;
+      ints = fixed;
+      err = dev_alloc((void**)&ctx->aux, ints * sizeof(int));
+    }
     if (err != cudaSuccess) return cuda_fail(err);
-    ctx->aux_ints = need;
+    ctx->aux_ints = ints;
   }
+  const size_t chain_ints = ((size_t)N + (size_t)pool) * kFrnnChunk;
   float4* emb_s = (float4*)ctx->aux;
   uint4* frag = (uint4*)(ctx->aux + 4 * (size_t)chunks * N);
   int* chains = (int*)frag + frag_ints;

@@ -93,6 +93,36 @@ def test_injected_allocation_failures_leave_context_usable():
 
 
 @pytest.mark.gpu
+def test_graph_building_goes_on_without_its_chunk_pool():
+    """A scratch that holds the chunks of hits with many partners does not fit: the build does without them, with the
+    same edges, and keeps that scratch; it fails when the rest does not fit either."""
+    import torch
+    from paper_2402_09633_gb300 import GnnError, InteractionNetwork
+    lib = _lib()
+    rng = np.random.default_rng(3)
+    emb = rng.standard_normal((3000, 8)).astype(np.float32)
+    emb = torch.from_numpy(emb / np.linalg.norm(emb, axis=1, keepdims=True)).cuda()
+    x = torch.rand(3000, 3, device="cuda")
+    blob = S.pack_blob(CFG, S.init_weights(CFG, 0))
+    net = InteractionNetwork(CFG, blob)
+    want = net.build_graph(emb, x, 0.8, 3000 * 1500)[0].cpu().numpy()
+    assert want.shape[1] > 15 * 3000                          # the average hit does not fit its first chunk
+    net.close()
+    net = InteractionNetwork(CFG, blob)
+    lib.gnn_debug_fail_allocs(2)
+    with pytest.raises(GnnError) as ex:
+        net.build_graph(emb, x, 0.8, 3000 * 1500)
+    assert ex.value.code == -3
+    for fails in (1, 0):                                       # the second call: with the scratch that is there
+        lib.gnn_debug_fail_allocs(fails)
+        got = net.build_graph(emb, x, 0.8, 3000 * 1500)[0].cpu().numpy()
+        assert lib.gnn_debug_fail_allocs(0) == 0 and got.tobytes() == want.tobytes()
+    small = net.build_graph(emb[:1000].contiguous(), x[:1000].contiguous(), 0.8, 1000 * 500)[0]
+    assert small.shape[1] > 1000
+    net.close()
+
+
+@pytest.mark.gpu
 def test_expired_device_wait_is_reported_and_context_stays_usable():
     import torch
     from paper_2402_09633_gb300 import InteractionNetwork
