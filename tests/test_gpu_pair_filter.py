@@ -70,6 +70,43 @@ def _unit(rng, n, dim):
     return (e / np.linalg.norm(e, axis=1, keepdims=True)).astype(np.float32)
 
 
+def pairs_at_the_radius(dim, scale, anchors, partners):
+    """Hits of length about `scale`, `partners` of them at a distance within 1e-6 of the radius from each anchor, on
+    either side; the radius."""
+    rng = np.random.default_rng(dim)
+    a = rng.standard_normal((anchors, dim))
+    a /= np.linalg.norm(a, axis=1, keepdims=True)
+    a = (a * scale).astype(np.float32)
+    radius = np.float32(0.08 * scale)
+    step = rng.standard_normal((anchors, partners, dim))
+    step /= np.linalg.norm(step, axis=2, keepdims=True)
+    b = a[:, None] + step * (radius * (1 + 1e-6 * rng.standard_normal((anchors, partners, 1))))
+    emb = np.concatenate([a, b.reshape(-1, dim).astype(np.float32)])
+    return np.ascontiguousarray(emb[rng.permutation(len(emb))]), radius
+
+
+def near_the_radius(emb, radius):
+    """How many pairs within the radius, and how many outside it, lie within 3e-6 of it."""
+    i, j = np.triu_indices(len(emb), 1)
+    d = np.sqrt(O.sq_dist_f32(emb[i], emb[j]).astype(np.float64))
+    near = np.abs(d / radius - 1) < 3e-6
+    inside = near & (O.sq_dist_f32(emb[i], emb[j]) < np.float32(radius * radius))
+    return inside.sum(), near.sum() - inside.sum()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dim", [3, 8, 16])
+@pytest.mark.parametrize("scale", [1e-3, 1.0, 37.0])
+def test_pairs_at_the_radius(dim, scale):
+    """The filter's margin on the GPU: thousands of pairs whose distance is the radius to a millionth."""
+    emb, radius = pairs_at_the_radius(dim, scale, 300, 12)
+    r = np.random.default_rng(0).random(len(emb)).astype(np.float32)
+    want = O.radius_graph(emb, r, radius)
+    inside, outside = near_the_radius(emb, radius)
+    assert inside > 1000 and outside > 1000
+    np.testing.assert_array_equal(_edges(emb, r, radius, 20 * len(emb)), want)
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n", [1, 2, 7, 8, 9, 15, 16, 17, 63, 64, 65, 700])
 @pytest.mark.parametrize("dim,radius", [(8, 0.9), (2, 0.05), (5, 0.3)])

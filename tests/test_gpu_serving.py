@@ -52,6 +52,72 @@ def test_cuda_graph_capture_and_replay():
     net.close()
 
 
+def test_capture_of_the_steps_around_the_network():
+    """The embedding, graph building, filter and track labels only enqueue kernels once their scratch is there: each
+    captured into a CUDA graph gives the eager outputs on new inputs of the same sizes, byte for byte."""
+    import ctypes
+    import torch
+    from paper_2402_09633_gb300 import InteractionNetwork
+    cfg = S.ModelConfig(12, 2, 64, 1, 2)
+    net = InteractionNetwork(cfg, S.pack_blob(cfg, S.init_weights(cfg, 5)))
+    net.load_embedding(S.pack_embed_blob(cfg, S.init_embed_weights(cfg, 8, 2)))
+    net.load_filter(S.pack_filter_blob(cfg, S.init_filter_weights(cfg, 3)))
+    n, m, room = 3000, 10007, 60000
+    xs, es = torch.zeros(n, 12, device="cuda"), torch.zeros(2, m, dtype=torch.int32, device="cuda")
+    emb = torch.zeros(n, 8, device="cuda")
+    score = torch.zeros(m, device="cuda")
+
+    def ints(*size):
+        return torch.zeros(*size, dtype=torch.int32, device="cuda")
+    edges, n_edges, kept, kept_id, n_kept, labels = ints(2 * room), ints(1), ints(2 * m), ints(m), ints(1), ints(n)
+    outs = {"embed": [emb], "graph": [n_edges, edges], "filter": [score, n_kept, kept, kept_id], "labels": [labels]}
+    p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    stream = torch.cuda.Stream()
+    st = ctypes.c_void_p(stream.cuda_stream)
+    calls = {
+        "embed": lambda: net.lib.gnn_embed(net.handle, p(xs), n, p(emb), st),
+        "graph": lambda: net.lib.gnn_build_graph(net.handle, p(emb), 8, p(xs), n, 0.3, room, p(edges), p(n_edges), st),
+        "filter": lambda: net.lib.gnn_filter_edges(net.handle, p(xs), p(es), n, m, 0.5, p(score), p(kept), p(kept_id),
+                                                   p(n_kept), st),
+        "labels": lambda: net.lib.gnn_track_labels(net.handle, p(score), p(es), n, m, 0.5, p(labels), st)}
+
+    def inputs(seed):
+        x, e = _event(seed)
+        assert x.shape == (n, 12) and e.shape == (2, m)
+        xs.copy_(torch.from_numpy(x)); es.copy_(torch.from_numpy(e))
+
+    def clear():
+        for t in (t for o in outs.values() for t in o):
+            t.zero_()
+        torch.cuda.synchronize()
+
+    def read():
+        torch.cuda.synchronize()
+        return {k: [t.cpu().numpy().tobytes() for t in o] for k, o in outs.items()}
+    inputs(0)
+    graphs = {}
+    for k, call in calls.items():
+        assert call() == 0                                     # eager first: the scratch is made here
+        stream.synchronize()
+        graphs[k] = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graphs[k], stream=stream):
+            assert call() == 0
+    for seed in (1, 0):
+        inputs(seed)
+        clear()
+        for call in calls.values():
+            assert call() == 0
+        want = read()
+        assert 0 < int(n_edges.item()) <= room and 0 < int(n_kept.item()) < m
+        clear()
+        for g in graphs.values():
+            g.replay()
+            torch.cuda.synchronize()
+        assert read() == want
+    assert net.status() == 0
+    net.close()
+
+
 def test_concurrent_contexts_on_separate_streams():
     """Several contexts (model instances) score different events on their own streams at the same
     time; each result equals its event scored alone."""

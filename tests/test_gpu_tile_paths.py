@@ -54,6 +54,35 @@ def test_tile_counts(tiles, last, L):
     check_parity(s, W, x, ei, cfg.n_iters)
 
 
+# The other models' regions and rings: H = 64 has five spare regions and eight stages, bf16 H = 128 streams the node
+# kernels' weights through four stages while the edge kernels' are resident.  Several rounds of tiles per group.
+@pytest.mark.parametrize("tiles,last", [(3 * 152 + 1, 1), (5 * 152, 64), (7 * 152 + 2, 127)])
+@pytest.mark.parametrize("H,bf16,L", [(64, False, 2), (64, False, 4), (64, True, 2), (64, True, 4), (128, True, 3),
+                                      (128, True, 4)])
+def test_tile_counts_of_the_other_models(tiles, last, H, bf16, L):
+    cfg = S.ModelConfig(3, 2, H, 1, L, S.PRECISION_BF16 if bf16 else S.PRECISION_FP32)
+    W = S.init_weights(cfg, 6)
+    n_edges = (tiles - 1) * 128 + last
+    x, ei = S.random_graph(n_edges // 2, n_edges, 3, seed=tiles)
+    s, rc = run_gpu(cfg, W, x, ei)
+    assert rc == 0
+    if not bf16:
+        check_parity(s, W, x, ei, cfg.n_iters)
+        return
+    # One iteration: an edge is either right to 1e-6 or some activation before it was rounded the other way, which
+    # 1 to 6 % of the edges see.  The 99th percentile then lies where that share begins and says little; compared with
+    # the oracle's float32 evaluation are the share itself, the mean error and the 99.9th percentile, each within 1.5
+    # times (0.88 to 1.2 over 24 graphs and weights), and no error beyond what one flipped rounding gives there.
+    _, z64 = O.forward(W, x, ei, 1, return_logits=True, bf16=True)
+    _, z32 = O.forward(W, x, ei, 1, return_logits=True, bf16=True, dtype=np.float32)
+    err, env = np.abs(logits_from_scores(s) - z64), np.abs(z32 - z64)
+    assert np.median(err) < 1e-6
+    assert np.mean(err > 1e-5) <= 1.5 * np.mean(env > 1e-5)
+    assert err.mean() <= 1.5 * env.mean()
+    assert np.percentile(err, 99.9) <= 1.5 * np.percentile(env, 99.9)
+    assert err.max() <= 3 * env.max()
+
+
 @pytest.mark.parametrize("feat", [2, 8, 9, 16])
 @pytest.mark.parametrize("H,L", [(128, 4), (64, 2)])
 def test_input_widths_of_encoder_and_filter(feat, H, L):

@@ -9,6 +9,7 @@ import pytest
 
 from oracle import gnn_oracle as O
 from tests import host_cuda
+from tests.test_gpu_pair_filter import near_the_radius, pairs_at_the_radius
 
 MAIN = r"""
 #include "ptx.cuh"
@@ -172,3 +173,15 @@ def test_single_hits_and_filter_agree(lib, dim):
     np.testing.assert_array_equal(ordered(want), O.radius_graph(emb, r, 0.05))
     for pool in (None, 0, 40):
         np.testing.assert_array_equal(build(lib, emb, r, 0.05, pool, single=True)[0], want)
+
+
+@pytest.mark.parametrize("dim", [3, 8, 12, 16])
+@pytest.mark.parametrize("scale", [1e-3, 1.0, 37.0])
+def test_pairs_at_the_radius(lib, dim, scale):
+    """Pairs whose distance is the radius to a millionth, with every error of the tensor core against them."""
+    emb, radius = pairs_at_the_radius(dim, scale, 30, 9)
+    r = np.random.default_rng(0).random(len(emb)).astype(np.float32)
+    want = O.radius_graph(emb, r, radius)
+    inside, outside = near_the_radius(emb, radius)
+    assert inside > 60 and outside > 60
+    np.testing.assert_array_equal(ordered(build(lib, emb, r, float(radius))[0]), want)
