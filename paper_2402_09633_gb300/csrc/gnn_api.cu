@@ -138,15 +138,16 @@ inline size_t swizzled_offset(int H, int n, int k) {
 void pack_block(const float* W, int ld, int col0, int H, bool with_lo, uint8_t* out) {
   const size_t part = (size_t)H * H * 2;
   for (int n = 0; n < H; ++n)
-    for (int k = 0; k < H; ++k) {
-      const float v = W[(size_t)n * ld + col0 + k];
-      const uint16_t hi = f32_to_bf16_rne(v);
-      const size_t off = swizzled_offset(H, n, k);
-      std::memcpy(out + off, &hi, 2);
-      if (with_lo) {
-        const uint16_t lo = f32_to_bf16_rne(v - bf16_to_f32(hi));
-        std::memcpy(out + part + off, &lo, 2);
+    for (int k0 = 0; k0 < H; k0 += 8) {              // a 16-byte unit of the layout
+      uint16_t hi[8], lo[8];
+      for (int k = 0; k < 8; ++k) {
+        const float v = W[(size_t)n * ld + col0 + k0 + k];
+        hi[k] = f32_to_bf16_rne(v);
+        lo[k] = f32_to_bf16_rne(v - bf16_to_f32(hi[k]));
       }
+      const size_t off = swizzled_offset(H, n, k0);
+      std::memcpy(out + off, hi, 16);
+      if (with_lo) std::memcpy(out + part + off, lo, 16);
     }
 }
 
@@ -174,12 +175,12 @@ void push(std::vector<float>& v, const float* p, size_t n) { v.insert(v.end(), p
 void centre_layer(const float* W, const float* b, int H, int in, std::vector<float>& Wc, std::vector<float>& bc) {
   Wc.resize((size_t)H * in);
   bc.resize(H);
-  for (int k = 0; k < in; ++k) {
-    double mu = 0.0;
-    for (int n = 0; n < H; ++n) mu += W[(size_t)n * in + k];
-    mu /= H;
-    for (int n = 0; n < H; ++n) Wc[(size_t)n * in + k] = (float)(W[(size_t)n * in + k] - mu);
-  }
+  std::vector<double> mu(in, 0.0);
+  for (int n = 0; n < H; ++n)
+    for (int k = 0; k < in; ++k) mu[k] += W[(size_t)n * in + k];
+  for (int k = 0; k < in; ++k) mu[k] /= H;
+  for (int n = 0; n < H; ++n)
+    for (int k = 0; k < in; ++k) Wc[(size_t)n * in + k] = (float)(W[(size_t)n * in + k] - mu[k]);
   double mb = 0.0;
   for (int n = 0; n < H; ++n) mb += b[n];
   mb /= H;
@@ -206,6 +207,7 @@ bool fold_gamma(std::vector<std::vector<float>*> W, std::vector<std::vector<floa
       const float a = std::fabs((*g[l])[i]);
       if (!(a >= 0.015625f && a <= 64.f)) return false;
     }
+  std::vector<float> scale((size_t)L * H);
   for (int l = 0; l + 1 < L; ++l)
     for (int i = 0; i < H; ++i) {
       const float s = (*g[l])[i] < 0.f ? -1.f : 1.f, a = std::fabs((*g[l])[i]);
@@ -213,8 +215,11 @@ bool fold_gamma(std::vector<std::vector<float>*> W, std::vector<std::vector<floa
       (*b[l])[i] *= s;
       (*be[l])[i] /= a;
       (*g[l])[i] = 1.f;
-      for (int n = 0; n < H; ++n) (*W[l + 1])[(size_t)n * in[l + 1] + i] *= a;
+      scale[l * H + i] = a;
     }
+  for (int l = 0; l + 1 < L; ++l)
+    for (int n = 0; n < H; ++n)
+      for (int i = 0; i < H; ++i) (*W[l + 1])[(size_t)n * in[l + 1] + i] *= scale[l * H + i];
   return true;
 }
 
@@ -249,23 +254,24 @@ void set_bias(KernelPlan& pl, int job, const float* b) {
 // the ones tile [128, 16] is (1, 1, 1, 0, ...); row n of a bias tile [H, 16] is b[n] in three bf16 parts
 // (24 bits, all of an fp32 value), then zeros.  K-major without a swizzle: element (r, k) at byte
 // (r / 8) * 256 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2.
-std::vector<uint8_t> const_tiles(const KernelPlan& pl, int H) {
-  std::vector<uint8_t> t(128 * 32 + pl.biases.size() * H * 32, 0);
-  auto put = [](uint8_t* tile, int r, int k, uint16_t v) {
-    std::memcpy(tile + (r / 8) * 256 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2, &v, 2);
+// Appended to `block`.
+void const_tiles(const KernelPlan& pl, int H, std::vector<uint8_t>& block) {
+  const size_t base = block.size();
+  block.resize(base + 128 * 32 + pl.biases.size() * H * 32, 0);
+  auto put = [&](size_t tile, int r, int k, uint16_t v) {
+    std::memcpy(block.data() + base + tile + (r / 8) * 256 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2, &v, 2);
   };
   for (int r = 0; r < 128; ++r)
-    for (int k = 0; k < 3; ++k) put(t.data(), r, k, f32_to_bf16_rne(1.0f));
+    for (int k = 0; k < 3; ++k) put(0, r, k, f32_to_bf16_rne(1.0f));
   for (size_t i = 0; i < pl.biases.size(); ++i)
     for (int n = 0; n < H; ++n) {
       float v = pl.biases[i][n];
       for (int k = 0; k < 3; ++k) {
         const uint16_t part = f32_to_bf16_rne(v);
-        put(t.data() + 128 * 32 + i * H * 32, n, k, part);
+        put(128 * 32 + i * H * 32, n, k, part);
         v -= bf16_to_f32(part);
       }
     }
-  return t;
 }
 
 // Every whole H-float segment of a plan's vector block is one per-column vector (bias, gamma,
@@ -300,15 +306,16 @@ cudaError_t dev_alloc(void** p, size_t bytes) {
 
 // A plan's vectors and constant tiles to the device.
 cudaError_t upload_plan(KernelPlan& pl, int H) {
-  const std::vector<uint8_t> tiles = const_tiles(pl, H);
-  pl.biases.clear();
   const size_t vb = (pl.vecs.size() * 4 + 255) & ~size_t(255);
-  pl.const_bytes = (uint32_t)tiles.size();
-  cudaError_t err = dev_alloc((void**)&pl.d_vecs, vb + tiles.size());
+  std::vector<uint8_t> block(vb, 0);
+  std::memcpy(block.data(), pl.vecs.data(), pl.vecs.size() * 4);
+  const_tiles(pl, H, block);
+  pl.biases.clear();
+  pl.const_bytes = (uint32_t)(block.size() - vb);
+  cudaError_t err = dev_alloc((void**)&pl.d_vecs, block.size());
   if (err != cudaSuccess) { pl.d_vecs = nullptr; return err; }
   pl.d_consts = (uint8_t*)pl.d_vecs + vb;
-  err = cudaMemcpy(pl.d_vecs, pl.vecs.data(), pl.vecs.size() * 4, cudaMemcpyHostToDevice);
-  if (err == cudaSuccess) err = cudaMemcpy(pl.d_consts, tiles.data(), tiles.size(), cudaMemcpyHostToDevice);
+  err = cudaMemcpy(pl.d_vecs, block.data(), block.size(), cudaMemcpyHostToDevice);
   return err;
 }
 
