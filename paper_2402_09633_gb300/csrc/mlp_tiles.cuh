@@ -18,7 +18,9 @@
 //
 // Organisation (one CTA per SM):
 //   * NG worker groups of eight warps: three for the edge kernels, the edge encoder, the filter and the
-//     embedding (80 registers a thread), two for the node kernels (120).  A group owns a tile at a time;
+//     embedding (72 registers a thread), two for the node kernels (96).  The issuing warp costs each worker
+//     registers: 25 warps put seven on one of the SM's four schedulers, 17 put five, and ptxas shares out
+//     its 16,384 registers by that.  The edge kernels spill 8 to 72 bytes at 72.  A group owns a tile at a time;
 //     a warp owns 16 rows of it, a quad of threads shares two rows (each thread a quarter of the
 //     columns), reads them from tensor memory with the 16-lane shapes and does the gathers, LayerNorm
 //     and ReLU in registers, in packed fp32 pairs;
@@ -43,7 +45,7 @@
 // epilogues and first layers on CUDA cores, fp32 / bf16 model: edge update 0.392 -> 0.288 / 0.313 -> 0.209
 // ms, node update 0.193 -> 0.163 / 0.140 -> 0.118, classifier 0.373 -> 0.262 / 0.331 -> 0.216, edge encoder
 // 0.284 -> 0.192 / 0.219 -> 0.150, node encoder 0.166 -> 0.114 / 0.139 -> 0.101; embedding of 300k hits
-// 0.204 -> 0.078, filter on 1.9M edges 0.90 -> 0.344.  Measured and not taken, in the edge update as it
+// 0.204 -> 0.078, filter on 1.9M edges 0.90 -> 0.344; the gammas' part in it is 0.5 to 0.8 % of a call.  Measured and not taken, in the edge update as it
 // was at 0.32 ms: one thread per row and four warps per group (every thread then reads every parameter:
 // 0.547 with shared memory, 0.371 through the constant cache); two groups with 104 registers (0.350);
 // gathers of one or three 32-column chunks before the layer-1 wait instead of two (0.328, 0.342).
@@ -79,7 +81,7 @@ __host__ __device__ constexpr bool has_input_job(TileKind k) {
 template <TileKind KIND>
 struct TileRoles {
   static constexpr int NG = (KIND == TileKind::NodeEncoder || KIND == TileKind::NodeUpdate) ? 2 : 3;
-  static constexpr int THREADS = 32 + 256 * NG;      // 800 (80 registers each) or 544 (120)
+  static constexpr int THREADS = 32 + 256 * NG;      // 800 (72 registers each) or 544 (96)
 };
 
 struct TileParams {
@@ -808,7 +810,7 @@ __global__ void __launch_bounds__(TileRoles<KIND>::THREADS, 1) mlp_tile_kernel(c
         GNN_TRACE_W(1);
         // layer-1 terms of the endpoints, loaded while the MMA runs: S = P_s[src] + P_d[dst] (P_d
         // carries b1), the first chunks before D is waited for, the others while those are added
-                constexpr int EARLY = NCH < 2 ? NCH : 2;
+        constexpr int EARLY = NCH < 2 ? NCH : 2;
         float2 S[NCH][8];
         auto gather = [&](int c) {
 #pragma unroll
